@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             ok = ok && wait(&sm.full[1], 0);
             if (ok) {
                 ptx::tc_fence_after();
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     const uint64_t w_desc = ptx::smem_desc(ptx::smem_addr(sm.codes[0]), kHalfBytes,
                                                            1024, ptx::kSwizzle128B);
                     const uint64_t q_desc =
@@ -532,7 +532,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             if (!wait(&sm.full[s], (u / kStages) & 1)) break;
             if (i >= 2 && !wait(&sm.s_empty[sb], ((i >> 1) - 1) & 1)) break;
             ptx::tc_fence_after();
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 const uint64_t a0 = c_desc + ((s * kCodeBytes) >> 4);
 #pragma unroll
                 for (int kk = 0; kk < kD / 32; ++kk)
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
             __syncwarp();
         }
-        if (lane == 0) ptx::mma_commit(&sm.drain);
+        if (ptx::elect_one()) ptx::mma_commit(&sm.drain);
         __syncwarp();
         const uint64_t t0 = ptx::globaltimer();
         while (!ptx::mbar_try_wait(&sm.drain, 0) && ptx::globaltimer() - t0 < kTimeoutNs) {
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             ptx::tc_fence_after();
             const int nvalid = min(kTile, t_end - (t_begin + j * kTile));
             const int ksteps = (nvalid + 31) >> 5;
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 const uint64_t a0 = c_desc + ((s * kCodeBytes) >> 4);
                 const uint64_t b0 = p_desc + ((pb * kPBytes) >> 4);
                 for (int kk = 0; kk < ksteps; ++kk)
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
             __syncwarp();
         }
-        if (lane == 0) ptx::mma_commit(&sm.drain2);
+        if (ptx::elect_one()) ptx::mma_commit(&sm.drain2);
         __syncwarp();
         const uint64_t t0 = ptx::globaltimer();
         while (!ptx::mbar_try_wait(&sm.drain2, 0) && ptx::globaltimer() - t0 < kTimeoutNs) {

@@ -788,7 +788,7 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
                 ok = wait(&sm.full[s], (r / NS) & 1);
                 if (!ok) break;
                 ptx::tc_fence_after();
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     const uint64_t w_desc = ptx::smem_desc(ptx::smem_addr(sm.tiles[s][0]), kHalfBytes,
                                                            1024, ptx::kSwizzle128B);
                     const uint32_t dst = route_pq ? tmem + 64 + 16 * r : tmem + 2 * kN;
@@ -811,7 +811,7 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
             if (!wait(&sm.full[s], ((i + ro) / NS) & 1)) break;
             if (i >= 2 && !wait(&sm.s_empty[sb], ((i >> 1) - 1) & 1)) break;
             ptx::tc_fence_after();
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 const uint64_t a0 = k_desc + ((s * kStageBytes) >> 4);
 #pragma unroll
                 for (int kk = 0; kk < kD / 16; ++kk) {
@@ -824,7 +824,7 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
             __syncwarp();
         }
         // Drain: every MMA this warp issued completes before TMEM is freed.
-        if (lane == 0) ptx::mma_commit(&sm.drain);
+        if (ptx::elect_one()) ptx::mma_commit(&sm.drain);
         __syncwarp();
         {
             const uint64_t t0 = ptx::globaltimer();
@@ -851,7 +851,7 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
             ptx::tc_fence_after();
             const int nvalid = min(kTile, t_end - (t_begin + j * kTile));
             const int ksteps = (nvalid + 15) >> 4;
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 const uint64_t a0 = v_desc + ((s * kStageBytes) >> 4);
                 const uint64_t b0 = p_desc + ((pb * kPBytes) >> 4);
                 for (int kk = 0; kk < ksteps; ++kk)
@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
             }
             __syncwarp();
         }
-        if (lane == 0) ptx::mma_commit(&sm.drain2);
+        if (ptx::elect_one()) ptx::mma_commit(&sm.drain2);
         __syncwarp();
         {
             const uint64_t t0 = ptx::globaltimer();

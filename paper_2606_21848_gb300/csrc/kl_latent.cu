@@ -152,7 +152,7 @@ __device__ void setup(LatentSmem &sm, int warp) {
 // Every MMA of the control warp has completed, all threads meet, TMEM is freed.
 __device__ void teardown(LatentSmem &sm, int warp, int lane) {
     if (warp == kCtlWarp) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             ptx::mma_commit(&sm.drain);
             settle(&sm.drain, 0);
         }
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool ok = wait_bar(sm, &sm.full, 0, err);
         if (ok) {
             ptx::tc_fence_after();
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 // Q_r = Q . W^R: A = Q (K-major), B = W^R (N = output dim, MN-major: halves kBox
                 // apart, 16 k rows = 2 KiB per step)
                 const uint64_t qd = ptx::smem_desc(ptx::smem_addr(q_s), 16, 1024, ptx::kSwizzle128B);
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (ok) {
             ptx::tc_fence_after();
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 // Q* = Q_hi . W_post^T + Q_lo . W_post^T: A = the pairs in TMEM (8 packed
                 // columns per step), B = W_post[h] (N = the r latent rows, K-major over D)
                 const uint64_t pd = ptx::smem_desc(ptx::smem_addr(sm.w), 16, 1024, ptx::kSwizzle128B);
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         ok = ok && wait_bar(sm, &sm.a_ready, 0, err);
         if (ok) {
             ptx::tc_fence_after();
-            if (lane == 0) {
+            if (ptx::elect_one()) {
                 // O = O*_hi . W_post + O*_lo . W_post: A = the pairs in TMEM, B = W_post[h]
                 // (N = output dim, MN-major: halves kBox apart, 16 latent rows = 2 KiB per step)
                 const uint64_t pd = ptx::smem_desc(ptx::smem_addr(sm.w), kBox, 1024, ptx::kSwizzle128B);

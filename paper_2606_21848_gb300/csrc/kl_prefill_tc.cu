@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = wait(&sm.full[0], 0);
             if (ok) {
                 ptx::tc_fence_after();
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     // Q_r = Q . W^R: A = query block (K-major), B = W^R (N = output dim j,
                     // MN-major)
 #pragma unroll
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (i >= 2 && !wait(&sm.s_free[sb], ((i >> 1) - 1) & 1)) { ok = false; break; }
                 if (!wait(&sm.full[s], (r / kStages) & 1)) { ok = false; break; }
                 ptx::tc_fence_after();
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     // S = Q_hi . V_i^T + Q_lo . V_i^T: A = Q_r in TMEM, B = the tile
                     // (N = tokens, K-major)
                     const uint64_t b0 = k_desc + ((s * kTileBytes) >> 4);
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const int s = (j + 1) % kStages;
                 if (!wait(&sm.p_full, j & 1)) { ok = false; break; }
                 ptx::tc_fence_after();
-                if (lane == 0) {
+                if (ptx::elect_one()) {
                     const uint64_t b0 = mn_desc + ((s * kTileBytes) >> 4);
                     const uint32_t pa = tmem + kColS + (j & 1) * 128u;
 #pragma unroll
@@ -383,7 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         (void)ok;
         // every MMA this warp issued completes before TMEM is freed
         uint64_t *drain = warp == kMmaWarp ? &sm.drain : &sm.drain2;
-        if (lane == 0) ptx::mma_commit(drain);
+        if (ptx::elect_one()) ptx::mma_commit(drain);
         __syncwarp();
         const uint64_t t0 = ptx::globaltimer();
         while (!ptx::mbar_try_wait(drain, 0) && ptx::globaltimer() - t0 < kTimeoutNs) {

@@ -13,6 +13,24 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// True in exactly one lane of the (converged) warp, the same one every time. The MMA issuers
+// branch on it rather than on lane == 0: their descriptors are warp-uniform operands, and behind
+// a branch that the compiler knows to hold one lane each tcgen05.mma issues in fewer cycles. Those
+// issue cycles are what the decode's small-N MMAs cost (group of 16 heads 252.9 -> 230.6 us, of
+// 32 248.3 -> 237.8 us, latent batch 98.5 -> 94.6 us, 70B batch 613.7 -> 604.2 us, chunked prefill
+// 595 -> 587 us; back-to-back calls). An issuer's commits must come from the same lane.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        :
+        : "memory");
+    return ok != 0;
+}
+
 // ------------------------------------------------------------------------- mbarrier ------
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count)
