@@ -17,6 +17,10 @@ cudaError_t launch_waits(const DecodeArgs &la, bool per_split, const CUtensorMap
 
 template <bool kStandard>
 cudaError_t launch(const DecodeArgs &a) {
+    // groups of more than 8 heads: one wide CTA per SM, unless the caller takes the split states
+    // (one per split) or the K+V comparison is asked for
+    if (!kStandard && a.geo.nhb > 1 && a.geo.D == 128 && (a.direct_out || a.merge_inside))
+        return launch_tc_wide(a);
     DecodeArgs la = a;
     const Geometry &g = la.geo;
     // cache viewed as [num_pages * Hkv * P rows][128]; one box = one page of one head

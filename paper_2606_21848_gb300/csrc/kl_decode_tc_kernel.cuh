@@ -280,11 +280,10 @@ __device__ __forceinline__ bool arrive_last(unsigned int *counter, int n) {
 // (kl_combine's formula). Up to eight splits: direct loads. More: the cache ring is idle by
 // now; the {m, l} table and the normalized weights go to its front, and TMA bulk copies bring
 // the state rows through the rest, folded by thread (head, 4 dims) from shared memory.
-template <int KH, int D, typename SmemT, typename WaitT>
+template <int kComputeWarps, int D, typename SmemT, typename WaitT>
 __device__ void merge_states(SmemT &sm, const DecodeArgs &a, int b, int qh0, int G, int n_u,
                              int t, int warp, int lane, const WaitT &wait) {
-    constexpr int kComputeWarps = Roles<KH>::kComputeWarps;
-    constexpr int kComputeThreads = Roles<KH>::kComputeThreads;
+    constexpr int kComputeThreads = kComputeWarps * 32;
     const Geometry &geo = a.geo;
     // a state row holds D floats: lanes below D / 4 fold them
     const bool lane_live = lane < D / 4;
@@ -336,7 +335,7 @@ __device__ void merge_states(SmemT &sm, const DecodeArgs &a, int b, int qh0, int
     }
     // Many splits: the {m, l} table and the weights go to the front of the idle ring, then the
     // state rows stream through the rest of it, `cap` splits per head per bulk-copy round.
-    uint8_t *ring = &sm.tiles[0][0][0];
+    uint8_t *ring = reinterpret_cast<uint8_t *>(sm.tiles);
     constexpr uint32_t kRingBytes = sizeof(sm.tiles);
     float2 *tab = reinterpret_cast<float2 *>(ring);                        // [G][n_u] {m, l}
     float *wt = reinterpret_cast<float *>(tab + G * n_u);                  // [G][n_u] weights
@@ -1252,7 +1251,8 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
                         sm.is_last = arrive_last(
                             a.counters + ((size_t)b * geo.Hkv + g) * geo.nhb + hb, n_cta_u) ? 1 : 0;
                     ptx::bar_sync(kBarCompute, kComputeThreads);
-                    if (sm.is_last) merge_states<KH, D>(sm, a, b, qh0, G, n_cta_u, tid, warp, lane, wait);
+                    if (sm.is_last)
+                        merge_states<kComputeWarps, D>(sm, a, b, qh0, G, n_cta_u, tid, warp, lane, wait);
                 }
             }
         }
@@ -1352,5 +1352,8 @@ cudaError_t launch_tc_head64(const DecodeArgs &la, bool per_split, bool standard
 cudaError_t launch_tc_groups(const DecodeArgs &la, bool per_split, bool standard, bool exact,
                              const CUtensorMap &vmap, const CUtensorMap &kmap,
                              const CUtensorMap &wmap, const CUtensorMap &qmap);
+// Groups of more than 8 heads at head dim 128 whose output this call writes (kl_decode_wide.cu):
+// up to 32 heads per CTA, one CTA per SM.
+cudaError_t launch_tc_wide(const DecodeArgs &a);
 
 }  // namespace kl

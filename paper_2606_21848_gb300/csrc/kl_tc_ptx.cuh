@@ -119,6 +119,24 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, u
         : "memory");
 }
 
+// The producers' page loop: lane p < 8 of the (converged) warp holds the row coordinate of page p
+// of a tile, `mask` the pages to load; one elected lane runs `load(p, row)` for each of them with
+// warp-uniform coordinates. TMA operands are uniform registers: issued by each page's own lane, a
+// tile of 8 pages (16 boxes) took 970 cycles, from one lane 306 (4 pages: 580 and 227).
+template <typename Begin, typename Load>
+__device__ __forceinline__ void for_pages(int row, unsigned mask, Begin &&begin, Load &&load) {
+    int r[8];
+#pragma unroll
+    for (int p = 0; p < 8; ++p) r[p] = __shfl_sync(0xffffffffu, row, p);
+    if (elect_one()) {
+        begin();
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            if (mask & (1u << p)) load(p, r[p]);
+    }
+    __syncwarp();
+}
+
 // 3-D tiled load of one box into shared memory, completing `bytes` on `bar`.
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar,
                                             int x, int y, int z) {
