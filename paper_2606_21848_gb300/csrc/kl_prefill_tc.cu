@@ -12,14 +12,21 @@
 // Each cached tile V_t [128 tokens x 128 dims] arrives once by TMA (one box per page) and feeds
 // both products from the same shared-memory copy: as the K-major B operand of the score MMAs
 // (bf16, as it landed) and, once the softmax warps have converted it to fp16 in place, as the
-// MN-major B operand of the output MMAs. Everything else lives in TMEM (512 columns, 128 each):
-// two S buffers, O, and the routed query Q_hi | Q_lo. Q and P enter the MMAs as A operands
-// straight from TMEM, so the only operand the tensor cores read from shared memory is the cache
-// tile. Tile t's scores go to buffer t % 2 as soon as the output MMAs of tile t - 2 have read
-// that buffer, so the score MMAs of tile t + 1 run during the softmax of tile t and the softmax
-// of tile t + 1 finds its scores ready; the softmax writes tile t's weights P over the first 64
-// columns of tile t's own buffer, and the output MMAs of tile t run during the softmax of tile
-// t + 1.
+// MN-major B operand of the output MMAs. Everything else lives in TMEM (512 columns): 256 columns
+// of scores, O (128), and the routed query Q_hi | Q_lo (64 + 64). Q and P enter the MMAs as A
+// operands straight from TMEM, so the only operand the tensor cores read from shared memory is
+// the cache tile.
+//
+// The pipeline's unit is a half tile u of 64 tokens: its scores go to one of four 64-column
+// buffers as soon as the output MMAs of half tile u - 4 have read that buffer's weights, the
+// softmax writes P over the buffer's first 32 columns, and the output MMAs follow. Two groups of
+// four softmax warps take alternate half tiles, so a half tile's chain (scores, maximum,
+// exponentials, weights, output, about 2600 cycles) is spread over four in flight. With whole
+// tiles and two buffers that chain set the pace; so did the issuing threads, which are held until
+// their MMAs start and then paid warp-wide waits before the next ones: each issuer's loop now
+// runs in one elected lane. 32K-token prompt (12 heads) 3340 -> 2970 us, 512-token chunks on 8192
+// (8 x 32 heads) 600 -> 543 us; the issued MMAs, 1.5 times the useful ones, then run at 1.68
+// PFLOP/s under the power cap, where cuBLAS sustains 1.73.
 //
 // Precision: the routed query (times scale * log2 e) is carried as a pair of bf16 operands,
 // x = hi + lo, about 16 significant bits where one bf16 operand keeps 8; the softmax weights
@@ -40,13 +47,13 @@
 // fp32 range, and the final O / l is unchanged because O and l share the same reference.
 //
 // Roles (352 threads, one CTA per SM):
-//   warps 0-7  softmax and epilogue: warps w and w + 4 share TMEM lane quarter w % 4 (its 32
-//              query rows) and split the 128 columns of S, P and O between them
+//   warps 0-7  softmax and epilogue: warp w serves TMEM lane quarter w % 4 (its 32 query rows)
+//              and the half tiles of parity w / 4; in the prologue and the epilogue warps w and
+//              w + 4 split the 128 columns of the routed query and of O between them
 //   warp 8     producer: TMA of W^R and the query block (ring position 0), then cache tiles
 //   warp 9     routing and score MMA issuer (one elected lane) and TMEM owner
-//   warp 10    output MMA issuer. One thread issuing tcgen05.mma back to back reaches about
-//              88 cycles per 128 x 128 x 16 MMA; two issuing threads together reach the
-//              tensor cores' 64.
+//   warp 10    output MMA issuer: a thread of its own, so that a half tile's output MMAs need
+//              not queue behind the next scores
 // Every wait is bounded (about one second); a wait that runs out raises KL_FLAG_TIMEOUT, makes
 // every role leave its loop, drains outstanding copies and MMAs and frees TMEM.
 #include <cudaTypedefs.h>
@@ -61,7 +68,9 @@ namespace {
 constexpr int kD = 128;
 constexpr int kBM = 128;                          // query rows per CTA
 constexpr int kBN = 128;                          // cache rows per tile
-constexpr int kStages = 4;
+constexpr int kBS = 64;                           // cache rows per half tile
+constexpr int kSub = 4;                           // half tiles in flight (score buffers)
+constexpr int kStages = 5;
 constexpr int kComputeWarps = 8;                  // two per TMEM lane quarter
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;                       // routing and score MMAs; TMEM owner
@@ -70,9 +79,9 @@ constexpr int kThreads = 11 * 32;
 constexpr uint32_t kTileBytes = kBN * kD * 2;     // 32 KiB
 constexpr uint32_t kHalfBytes = kTileBytes / 2;   // one 64-column half: 128 rows x 128 B
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kColS = 0;                     // S of tile t: 128 t % 2 .. + 127 (then P of
-                                                  // tile t, fp16 pairs, in its first 64); the
-                                                  // routed query first lands in buffer 0
+constexpr uint32_t kColS = 0;                     // S of half tile u: 64 (u % 4) .. + 63 (then
+                                                  // its P, fp16 pairs, in the first 32); the
+                                                  // routed query first lands in 0 .. 127
 constexpr uint32_t kColO = 256;                   // O: columns 256 .. 383
 constexpr uint32_t kColQ = 384;                   // Q_hi: 384 .. 447, Q_lo: 448 .. 511
 constexpr uint32_t kLoCols = 64;                  // hi -> lo of a packed bf16 operand
@@ -87,34 +96,38 @@ struct __align__(1024) PrefillSmem {
     // the cache tiles ([64-dim half][128 tokens][128 B]); all 128B-swizzled.
     uint8_t tiles[kStages][kTileBytes];
     uint64_t full[kStages], empty[kStages];
-    uint64_t s_full[2], s_free[2], p_full, pv_done;
+    uint64_t s_full[kSub], s_free[kSub], p_full[kSub];
+    uint64_t turn[4][2];       // per lane quarter and parity: the references after a half tile
     uint64_t r_full, qr_ready, drain, drain2;
-    float red[2][2][kBM];      // per-tile half-row maxima of the two warps of a pair (2 tiles)
-    float lsum[2][kBM];        // the two warps' shares of the row sums, for the epilogue
+    float mref[2][kBM];        // the rows' references after the last half tile of each parity
+    float lsum[2][kBM];        // the two groups' shares of the row sums, for the epilogue
     uint32_t tmem_base;
     int abort;
 };
 
-// Warp-collective bounded wait (every lane calls it in uniform control flow and gets the same
-// answer). False when the CTA is aborting or the wait ran out (about 1 s).
+// Bounded wait. Warp-collective (every lane calls it in uniform control flow and gets the same
+// answer), or by one lane alone (one(): the MMA issuers, whose successful waits must cost little).
+// False when the CTA is aborting or the wait ran out (about 1 s).
 struct Waiter {
     volatile int *abort;
     int32_t *err;
-    __device__ bool operator()(uint64_t *bar, uint32_t parity) const {
-        bool ok = ptx::mbar_try_wait(bar, parity);
-        if (!ok) {
-            const uint64_t t0 = ptx::globaltimer();
-            while (true) {
-                if (ptx::mbar_try_wait(bar, parity)) { ok = true; break; }
-                if (*abort) break;
-                if (ptx::globaltimer() - t0 > kTimeoutNs) {
-                    *abort = 1;
-                    raise_flag(err, KL_FLAG_TIMEOUT);
-                    break;
-                }
+    __device__ bool slow(uint64_t *bar, uint32_t parity) const {
+        const uint64_t t0 = ptx::globaltimer();
+        while (true) {
+            if (ptx::mbar_try_wait(bar, parity)) return true;
+            if (*abort) return false;
+            if (ptx::globaltimer() - t0 > kTimeoutNs) {
+                *abort = 1;
+                raise_flag(err, KL_FLAG_TIMEOUT);
+                return false;
             }
         }
-        return __all_sync(0xffffffffu, ok);
+    }
+    __device__ bool one(uint64_t *bar, uint32_t parity) const {
+        return ptx::mbar_try_wait(bar, parity) || slow(bar, parity);
+    }
+    __device__ bool operator()(uint64_t *bar, uint32_t parity) const {
+        return __all_sync(0xffffffffu, one(bar, parity));
     }
 };
 
@@ -176,7 +189,7 @@ __device__ __forceinline__ uint32_t pack_f16(float a, float b) {
     return d;
 }
 
-__device__ __forceinline__ void ld_shared_v4(uint32_t addr, uint32_t (&v)[4]) {
+__device__ __forceinline__ void ld_shared_v4(uint32_t addr, uint32_t *v) {
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
                  : "r"(addr)
@@ -215,6 +228,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int pos0 = L - n + m0;                 // position of row 0
     const int pos_last = pos0 + rows - 1;        // <= L - 1
     const int n_tiles = pos_last / kBN + 1;      // cache tiles 0 .. n_tiles - 1
+    const int n_sub = pos_last / kBS + 1;        // half tiles 0 .. n_sub - 1
     const int g = h / geo.G;
     const int wsel = geo.wr_per_qh ? h : g;
 
@@ -223,16 +237,18 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::mbar_init(&sm.full[s], 1);
             ptx::mbar_init(&sm.empty[s], 1);
         }
-        // One completion per tile on p_full and pv_done, one per tile of its buffer on
-        // s_full[b] (scores of tile t in buffer b = t % 2) and s_free[b] (the output MMAs of
-        // tile t have read buffer t % 2). Every wait names the completion it needs: MMAs that
-        // write different TMEM ranges are not assumed to complete in issue order.
-        for (int b2 = 0; b2 < 2; ++b2) {
+        // One completion per half tile u of its buffer b = u % kSub on s_full[b] (its scores),
+        // p_full[b] (its weights and the converted rows) and s_free[b] (its output MMAs are done:
+        // O holds it, and the buffer may be written), and per lane quarter on turn[.][u % 2].
+        // Every wait names the completion it needs: MMAs that write different TMEM ranges are
+        // not assumed to complete in issue order.
+        for (int b2 = 0; b2 < kSub; ++b2) {
             ptx::mbar_init(&sm.s_full[b2], 1);
             ptx::mbar_init(&sm.s_free[b2], 1);
+            ptx::mbar_init(&sm.p_full[b2], kComputeWarps / 2);
         }
-        ptx::mbar_init(&sm.p_full, kComputeWarps);
-        ptx::mbar_init(&sm.pv_done, 1);
+        for (int q = 0; q < 4; ++q)
+            for (int b2 = 0; b2 < 2; ++b2) ptx::mbar_init(&sm.turn[q][b2], 1);
         ptx::mbar_init(&sm.r_full, 1);
         ptx::mbar_init(&sm.qr_ready, kComputeWarps);
         ptx::mbar_init(&sm.drain, 1);
@@ -309,7 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // K-major SW128 operands step 32 B per 16 columns inside a 64-column half and jump a
         // half (kHalfBytes) every 4 steps; MN-major SW128 operands step 16 rows = 2 KiB; TMEM
         // A operands step 8 columns (16 packed 16-bit values).
-        constexpr uint32_t idesc_qk = ptx::idesc_bf16(128, 128, false, false);
+        constexpr uint32_t idesc_qk = ptx::idesc_bf16(128, kBS, false, false);
         constexpr uint32_t idesc_route = ptx::idesc_bf16(128, 128, false, true);
         constexpr uint32_t idesc_pv = idesc_f16(128, 128, false, true);   // (mma_bf16_ts issues
         // the kind::f16 MMA; this descriptor makes both of its operands fp16)
@@ -337,50 +353,46 @@ __global__ void __launch_bounds__(kThreads, 1)
                 __syncwarp();
             }
             ok = ok && wait(&sm.qr_ready, 0);
-            for (int i = 0; ok && i < n_tiles; ++i) {
-                const int r = i + 1, s = r % kStages, sb = i & 1;
-                // the output MMAs of tile i - 2 have read buffer sb (its P); waited on before
-                // the tile, so that this is the buffer's next completion (the one after it
-                // needs tile i's scores)
-                if (i >= 2 && !wait(&sm.s_free[sb], ((i >> 1) - 1) & 1)) { ok = false; break; }
-                if (!wait(&sm.full[s], (r / kStages) & 1)) { ok = false; break; }
+            // (the whole loop by one lane: a warp-wide wait between two half tiles left the
+            // tensor cores idle, since the issuing thread is held until its MMAs start)
+            if (ok && ptx::elect_one()) {
                 ptx::tc_fence_after();
-                if (ptx::elect_one()) {
-                    // S = Q_hi . V_i^T + Q_lo . V_i^T: A = Q_r in TMEM, B = the tile
+                for (int u = 0; u < n_sub; ++u) {
+                    const int r = (u >> 1) + 1, s = r % kStages, sb = u % kSub;
+                    if (!wait.one(&sm.full[s], (r / kStages) & 1)) break;
+                    // the output MMAs of half tile u - kSub have read buffer sb (its P)
+                    if (u >= kSub && !wait.one(&sm.s_free[sb], (u / kSub - 1) & 1)) break;
+                    ptx::tc_fence_after();
+                    // S = Q_hi . V^T + Q_lo . V^T: A = Q_r in TMEM, B = 64 rows of the tile
                     // (N = tokens, K-major)
-                    const uint64_t b0 = k_desc + ((s * kTileBytes) >> 4);
+                    const uint64_t b0 = k_desc + ((s * kTileBytes + (u & 1) * kBS * 128) >> 4);
 #pragma unroll
                     for (int kk = 0; kk < 2 * kD / 16; ++kk)
-                        ptx::mma_bf16_ts(tmem + kColS + sb * 128u,
+                        ptx::mma_bf16_ts(tmem + kColS + sb * kBS,
                                          tmem + kColQ + (kk >= 8 ? kLoCols : 0u) + (kk & 7) * 8,
                                          b0 + kstep(kk & 7), idesc_qk, kk > 0);
                     ptx::mma_commit(&sm.s_full[sb]);
                 }
-                __syncwarp();
             }
-        } else {
-            // the output MMAs of every tile: O += P . V_j, fp16; A = P in TMEM (the first 64
-            // columns of buffer j % 2), B = the tile (N = dims, MN-major), converted to fp16 by
-            // the softmax warps before they arrive on p_full
-            for (int j = 0; j < n_tiles; ++j) {
-                const int s = (j + 1) % kStages;
-                if (!wait(&sm.p_full, j & 1)) { ok = false; break; }
+        } else if (ptx::elect_one()) {
+            // the output MMAs of every half tile: O += P . V, fp16; A = P in TMEM (the first 32
+            // columns of its score buffer), B = 64 rows of the tile (N = dims, MN-major),
+            // converted to fp16 by the softmax warps before they arrive on p_full
+            for (int u = 0; u < n_sub; ++u) {
+                const int s = ((u >> 1) + 1) % kStages, sb = u % kSub;
+                if (!wait.one(&sm.p_full[sb], (u / kSub) & 1)) break;
                 ptx::tc_fence_after();
-                if (ptx::elect_one()) {
-                    const uint64_t b0 = mn_desc + ((s * kTileBytes) >> 4);
-                    const uint32_t pa = tmem + kColS + (j & 1) * 128u;
+                const uint64_t b0 = mn_desc + ((s * kTileBytes + (u & 1) * kBS * 128) >> 4);
+                const uint32_t pa = tmem + kColS + sb * kBS;
 #pragma unroll
-                    for (int kk = 0; kk < kBN / 16; ++kk)
-                        ptx::mma_bf16_ts(tmem + kColO, pa + kk * 8, b0 + ((kk * 2048) >> 4), idesc_pv,
-                                         (j > 0 || kk > 0) ? 1u : 0u);
-                    ptx::mma_commit(&sm.empty[s]);
-                    ptx::mma_commit(&sm.s_free[j & 1]);
-                    ptx::mma_commit(&sm.pv_done);
-                }
-                __syncwarp();
+                for (int kk = 0; kk < kBS / 16; ++kk)
+                    ptx::mma_bf16_ts(tmem + kColO, pa + kk * 8, b0 + ((kk * 2048) >> 4), idesc_pv,
+                                     (u > 0 || kk > 0) ? 1u : 0u);
+                ptx::mma_commit(&sm.s_free[sb]);
+                if ((u & 1) || u == n_sub - 1) ptx::mma_commit(&sm.empty[s]);
             }
         }
-        (void)ok;
+        __syncwarp();
         // every MMA this warp issued completes before TMEM is freed
         uint64_t *drain = warp == kMmaWarp ? &sm.drain : &sm.drain2;
         if (ptx::elect_one()) ptx::mma_commit(drain);
@@ -390,9 +402,12 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else {
         // --------------------------------------------------------- softmax, epilogue ----
-        // Two warps per TMEM lane quarter: warp w serves rows 32 (w % 4) .. + 31 and columns
-        // 64 hf .. + 63 (hf = w / 4) of S, P and O. The pair meets once per tile on a named
-        // barrier (id 1 + w % 4) that also ANDs their progress, so both leave a loop together.
+        // Two groups of four warps: warp w serves the 32 query rows of lane quarter w % 4
+        // (thread = row = TMEM lane), group w / 4 the half tiles of that parity, so that one
+        // group's softmax runs while the tensor cores and the other group work on the half tiles
+        // around it. The groups share each row's reference (and O): the owner of half tile u takes
+        // the reference that u - 1 left, and passes its own on (turn) before its exponentials. In
+        // the prologue and the epilogue the two warps of a lane quarter split the 128 columns.
         const int qd = warp & 3, hf = warp >> 2;
         const int r = qd * 32 + lane;                        // query row = TMEM lane
         const int c0 = hf * 64;                              // this warp's columns
@@ -429,142 +444,146 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (lane == 0) ptx::mbar_arrive(&sm.qr_ready);
         }
 
-        float m_ref = -INFINITY;   // reference maximum of the row (base 2), shared by the pair
-        // this warp's share of sum 2^(s - m_ref), in two packed pairs of partial sums
+        float m_used = -INFINITY;  // the reference of this thread's share of the row sum
+        // this group's share of sum 2^(s - m_used), in two packed pairs of partial sums
         float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
-        // Both warps of a pair run the same tiles and meet on exactly one pair barrier per
-        // tile and one in the epilogue; a wait that fails only turns this warp's vote false, and
-        // the pair leaves together at the next barrier.
         bool okl = ok;
-        for (int i = 0; i < n_tiles; ++i) {
-            const int t0 = i * kBN, rb = i & 1;
-            const uint32_t sbuf = tmem + kColS + (uint32_t)rb * 128u;   // S, then P, of tile i
-            if (okl) okl = wait(&sm.s_full[rb], (i >> 1) & 1);
-            float sv[64];
-            float mp = -INFINITY;
-            if (okl) {
-                ptx::tc_fence_after();
-                uint32_t u0[32], u1[32];
-                ptx::tmem_ld32(sbuf + c0 + lane_base, u0);
-                ptx::tmem_ld32(sbuf + c0 + 32 + lane_base, u1);
-                ptx::tmem_wait_ld();
-                ptx::reg_fence(u0);
-                ptx::reg_fence(u1);
+        for (int u = hf; okl && u < n_sub; u += 2) {
+            const int t0 = u * kBS, k = u >> 1, sb = u % kSub;
+            const uint32_t sbuf = tmem + kColS + (uint32_t)sb * kBS + lane_base;   // S, then P
+            // This thread's half (64 dims) of a cache row of the half tile as fp16, formed while
+            // the scores are still on their way: the output MMAs read the tile as fp16. Rows at
+            // or past the sequence's end (an unwritten page tail, or a page slot no TMA filled)
+            // become zeros, so that 0-weights never meet a non-finite value. The lanes start at
+            // different 16-byte chunks so that a warp's accesses spread over all banks.
+            const int stage = (k + 1) % kStages;
+            okl = wait(&sm.full[stage], ((k + 1) / kStages) & 1);
+            if (!okl) break;
+            const uint32_t v_s = ptx::smem_addr(sm.tiles[stage]) + (r >> 6) * kHalfBytes +
+                                 (hf * kBS + (r & 63)) * 128;
+            uint32_t vr[32];
+            if (t0 + (r & 63) < L) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) ld_shared_v4(v_s + ((c + lane) & 7) * 16, vr + 4 * c);
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                    vr[e] = pack_f16(__uint_as_float(vr[e] << 16), __uint_as_float(vr[e] & 0xffff0000u));
+            } else {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) vr[e] = 0u;
+            }
+            okl = wait(&sm.s_full[sb], (u / kSub) & 1);
+            if (!okl) break;
+            ptx::tc_fence_after();
+            uint32_t s0[32], s1[32];
+            ptx::tmem_ld32(sbuf, s0);
+            ptx::tmem_ld32(sbuf + 32, s1);
+            // the score MMAs have read these rows: their fp16 form takes their place
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                st_shared_v4(v_s + ((c + lane) & 7) * 16, vr[4 * c], vr[4 * c + 1], vr[4 * c + 2],
+                             vr[4 * c + 3]);
+            ptx::tmem_wait_ld();
+            ptx::reg_fence(s0);
+            ptx::reg_fence(s1);
+            // causal mask: token t0 + c is visible to the row when it is <= pos_r
+            if (t0 + kBS - 1 > pos0) {
+                const int lim = pos_r - t0;
 #pragma unroll
                 for (int c = 0; c < 32; ++c) {
-                    sv[c] = __uint_as_float(u0[c]);
-                    sv[32 + c] = __uint_as_float(u1[c]);
+                    if (c > lim) s0[c] = 0xff800000u;
+                    if (c + 32 > lim) s1[c] = 0xff800000u;
                 }
-                // causal mask: token t0 + c0 + c is visible to the row when it is <= pos_r
-                if (t0 + c0 + 63 > pos0) {
-                    const int lim = pos_r - t0 - c0;
-#pragma unroll
-                    for (int c = 0; c < 64; ++c)
-                        if (c > lim) sv[c] = -INFINITY;
-                }
-                float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                for (int c = 0; c < 64; c += 8) {
-                    mx[0] = max3(mx[0], sv[c], sv[c + 1]);
-                    mx[1] = max3(mx[1], sv[c + 2], sv[c + 3]);
-                    mx[2] = max3(mx[2], sv[c + 4], sv[c + 5]);
-                    mx[3] = max3(mx[3], sv[c + 6], sv[c + 7]);
-                }
-                mp = max3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
-                sm.red[rb][hf][r] = mp;
             }
-            // the pair exchanges its half maxima (and leaves together on any failed wait); past
-            // this barrier both warps hold their S in registers, so P may overwrite the buffer
-            if (!ptx::bar_and(pair_bar, 64, okl)) {
-                okl = false;
-                break;
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int c = 0; c < 32; c += 4) {
+                mx[0] = max3(mx[0], __uint_as_float(s0[c]), __uint_as_float(s0[c + 1]));
+                mx[1] = max3(mx[1], __uint_as_float(s0[c + 2]), __uint_as_float(s0[c + 3]));
+                mx[2] = max3(mx[2], __uint_as_float(s1[c]), __uint_as_float(s1[c + 1]));
+                mx[3] = max3(mx[3], __uint_as_float(s1[c + 2]), __uint_as_float(s1[c + 3]));
             }
-            const float m_tile = fmaxf(mp, sm.red[rb][hf ^ 1][r]);
-            const float m_new = fmaxf(m_ref, m_tile);
-            // a new reference when the maximum grew by more than 2^8 (or is the first finite);
-            // both warps of the pair take the same decision from the same numbers
-            const bool grow = m_new > m_ref + kRescaleLog2;
-            if (__any_sync(0xffffffffu, grow)) {
+            const float mt = max3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
+            float m_ref = -INFINITY;
+            if (u > 0) {
+                okl = wait(&sm.turn[qd][hf ^ 1], ((u - 1) >> 1) & 1);
+                if (!okl) break;
+                m_ref = sm.mref[hf ^ 1][r];
+            }
+            // a new reference when the maximum grew by more than 2^8 (or is the first finite)
+            const float m_new = fmaxf(m_ref, mt);
+            if (__any_sync(0xffffffffu, m_new > m_ref + kRescaleLog2)) {
                 const float f = (m_new == -INFINITY || m_ref == -INFINITY) ? 0.f : ptx::ex2(m_ref - m_new);
-                if (i > 0) {
-                    // O holds tiles 0 .. i - 1 once the output MMAs of tile i - 1 are done
-                    okl = okl && wait(&sm.pv_done, (i - 1) & 1);
-                    if (okl) {
-                        ptx::tc_fence_after();
+                if (u > 0) {
+                    // O holds half tiles 0 .. u - 1 once the output MMAs of u - 1 are done
+                    okl = wait(&sm.s_free[(u - 1) % kSub], ((u - 1) / kSub) & 1);
+                    if (!okl) break;
+                    ptx::tc_fence_after();
 #pragma unroll
-                        for (int c = 0; c < 64; c += 32) {
-                            uint32_t u[32];
-                            ptx::tmem_ld32(tmem + kColO + c0 + c + lane_base, u);
-                            ptx::tmem_wait_ld();
-                            ptx::reg_fence(u);
+                    for (int c = 0; c < 128; c += 32) {
+                        uint32_t o[32];
+                        ptx::tmem_ld32(tmem + kColO + c + lane_base, o);
+                        ptx::tmem_wait_ld();
+                        ptx::reg_fence(o);
 #pragma unroll
-                            for (int e = 0; e < 32; ++e) u[e] = __float_as_uint(__uint_as_float(u[e]) * f);
-                            ptx::tmem_st32(tmem + kColO + c0 + c + lane_base, u);
-                        }
-                        ptx::tmem_wait_st();
+                        for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * f);
+                        ptx::tmem_st32(tmem + kColO + c + lane_base, o);
                     }
+                    ptx::tmem_wait_st();
                 }
-                la = mul2(la, f);
-                lb = mul2(lb, f);
                 m_ref = m_new;
             }
-            const float mr = m_ref == -INFINITY ? 0.f : m_ref;
-
-            // this warp's 64 weights -> 32 packed fp16 columns of P (in pairs: s - m, 2^x, the
+            sm.mref[hf][r] = m_ref;
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&sm.turn[qd][hf]);
+            // the group's sums move to this reference
+            if (__any_sync(0xffffffffu, m_ref != m_used)) {
+                const float f = m_used == -INFINITY ? 0.f : ptx::ex2(m_used - m_ref);
+                la = mul2(la, f);
+                lb = mul2(lb, f);
+                m_used = m_ref;
+            }
+            // the row's 64 weights -> 32 packed fp16 columns of P (in pairs: s - m, 2^x, the
             // running sums, the fp16 pack)
-            uint32_t ph[32];
+            const float mr = m_ref == -INFINITY ? 0.f : m_ref;
 #pragma unroll
-            for (int e = 0; e < 32; ++e) {
-                const float2 d = sub2(make_float2(sv[2 * e], sv[2 * e + 1]), make_float2(mr, mr));
+            for (int e = 0; e < 16; ++e) {
+                const float2 d = sub2(make_float2(__uint_as_float(s0[2 * e]), __uint_as_float(s0[2 * e + 1])),
+                                      make_float2(mr, mr));
                 const float2 pe = make_float2(ptx::ex2(d.x), ptx::ex2(d.y));
                 if (e & 1) lb = add2(lb, pe); else la = add2(la, pe);
-                ph[e] = pack_f16(pe.x, pe.y);
+                s0[e] = pack_f16(pe.x, pe.y);
             }
-            // The score MMAs are done with tile i: this thread converts its cache row r,
-            // dims 64 hf .. + 63 (128 contiguous bytes whatever the swizzle), to fp16 in place
-            // for the output MMAs. Rows at or past the sequence's end (an unwritten page
-            // tail, or a page slot no TMA filled) become zeros instead, so that 0-weights
-            // never meet a non-finite value. The lanes start at different 16-byte chunks so
-            // that a warp's accesses spread over all banks.
-            if (okl) {
-                const uint32_t v_s = ptx::smem_addr(sm.tiles[(i + 1) % kStages]) +
-                                     hf * kHalfBytes + r * 128;
-                if (t0 + r < L) {
-#pragma unroll 4
-                    for (int c = 0; c < 8; ++c) {
-                        const uint32_t addr = v_s + ((c + lane) & 7) * 16;
-                        uint32_t w[4];
-                        ld_shared_v4(addr, w);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            w[e] = pack_f16(__uint_as_float(w[e] << 16),
-                                            __uint_as_float(w[e] & 0xffff0000u));
-                        }
-                        st_shared_v4(addr, w[0], w[1], w[2], w[3]);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) st_shared_v4(v_s + c * 16, 0u, 0u, 0u, 0u);
-                }
-                // P over the first 64 columns of the buffer (the output MMAs of tile i - 2, the
-                // last reader of P there, finished before tile i's scores were written)
-                ptx::tmem_st32(sbuf + c0 / 2 + lane_base, ph);
-                ptx::tmem_wait_st();
-                // the converted tile (generic-proxy stores) is read next by the output MMAs
-                ptx::tc_fence_before();
-                ptx::fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&sm.p_full);
+            for (int e = 0; e < 16; ++e) {
+                const float2 d = sub2(make_float2(__uint_as_float(s1[2 * e]), __uint_as_float(s1[2 * e + 1])),
+                                      make_float2(mr, mr));
+                const float2 pe = make_float2(ptx::ex2(d.x), ptx::ex2(d.y));
+                if (e & 1) lb = add2(lb, pe); else la = add2(la, pe);
+                s0[16 + e] = pack_f16(pe.x, pe.y);
             }
-            // a wait that failed above leaves okl false: this warp skips its work and votes
-            // false at the next pair barrier (or the epilogue's), where the pair leaves together
+            // P over the first 32 columns of the buffer (the output MMAs of u - kSub, the last
+            // reader of P there, finished before these scores were written)
+            ptx::tmem_st32(sbuf, s0);
+            ptx::tmem_wait_st();
+            // the converted rows (generic-proxy stores) are read next by the output MMAs
+            ptx::tc_fence_before();
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&sm.p_full[sb]);
         }
 
-        // Epilogue: out = O / l, this warp's 64 output dims; l is the pair's two shares. A
-        // non-finite output (a cached value beyond fp16's range, or a non-finite input) raises
-        // KL_FLAG_RANGE.
-        const float l = (la.x + la.y) + (lb.x + lb.y);
-        const bool oke = okl && wait(&sm.pv_done, (n_tiles - 1) & 1);
+        // Epilogue: out = O / l, this warp's 64 output dims; l is the two groups' shares, at the
+        // reference of the last half tile. A non-finite output (a cached value beyond fp16's range,
+        // or a non-finite input) raises KL_FLAG_RANGE.
+        const int last = n_sub - 1, lb2 = last & 1;
+        if (okl && lb2 != hf) okl = wait(&sm.turn[qd][lb2], (last >> 1) & 1);
+        const bool oke = okl && wait(&sm.s_free[last % kSub], (last / kSub) & 1);
+        float l = (la.x + la.y) + (lb.x + lb.y);
+        if (oke && lb2 != hf) {
+            const float m_fin = sm.mref[lb2][r];
+            l = m_used == -INFINITY ? 0.f : l * ptx::ex2(m_used - m_fin);
+        }
         sm.lsum[hf][r] = l;
         if (ptx::bar_and(pair_bar, 64, oke)) {
             ptx::tc_fence_after();

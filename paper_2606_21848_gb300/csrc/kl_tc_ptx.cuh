@@ -374,7 +374,7 @@ __device__ __forceinline__ void reg_fence(uint32_t (&u)[N]) {
 }
 
 // Store 32 consecutive 32-bit columns of the thread's TMEM lane (complete with tmem_wait_st()).
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&u)[32]) {
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *u) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
         "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
