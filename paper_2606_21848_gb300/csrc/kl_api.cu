@@ -197,7 +197,7 @@ kl_status decode_common(bool standard, const kl_shape *shape, const void *q, con
 cudaError_t finish_decode(const DecodeArgs &a, bool states_requested) {
     if (a.direct_out || a.merge_inside || states_requested) return cudaSuccess;
     return launch_combine(a.geo.B, a.geo.Hq, a.geo.D, a.geo.S, a.part_o, a.part_ml, a.out,
-                          a.out_dtype, a.stream, true);
+                          a.out_dtype, a.stream);
 }
 
 }  // namespace kl

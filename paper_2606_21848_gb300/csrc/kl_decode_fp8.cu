@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     decode_fp8_kernel(const __grid_constant__ CUtensorMap cmap,
                       const __grid_constant__ CUtensorMap wmap,
                       const __grid_constant__ CUtensorMap qmap, const DecodeArgs a,
-                      const float *__restrict__ v_scales) {
+                      const float *v_scales) {
     using Sh = Fp8Shape<KHH>;
     extern __shared__ uint8_t smem_raw[];
     // kAllLive: the group has 2 KHH heads, so no compute warp holds a padded head
@@ -330,11 +330,6 @@ __global__ void __launch_bounds__(kThreads, 2)
     const bool route = a.w_r != nullptr;      // W^R given; else q is the composed query
     // Ring uses: with routing, uses 0 and 1 are the W^R halves and tile i is use i + 2.
     const int base = route ? 2 : 0;
-
-    const int L_raw = a.seq_lens[b];
-    const int pos_raw = a.v_new ? a.positions[b] : -1;
-    const int t_begin = split * geo.chunk;
-    const int32_t *bt = a.block_table + (size_t)b * geo.max_pages;
 
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -367,11 +362,17 @@ __global__ void __launch_bounds__(kThreads, 2)
             ptx::prefetch_tensormap(&qmap);
         }
     }
+    grid_dep_wait();        // nothing above touched global memory
+    const int L_raw = a.seq_lens[b];
+    const int pos_raw = a.v_new ? a.positions[b] : -1;
+    const int t_begin = split * geo.chunk;
+    const int32_t *bt = a.block_table + (size_t)b * geo.max_pages;
+
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    // the combine of the split states, launched behind as a programmatic dependent, may start
-    // setting up once every CTA is here
+    // the kernel behind (the combine of the split states, the next call) may start setting up once
+    // every CTA is here
     grid_dep_launch();
 
     int L = L_raw;
@@ -975,6 +976,7 @@ cudaError_t launch_shape(const DecodeArgs &a, const CUtensorMap &cmap, const CUt
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = a.stream;
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, decode_fp8_kernel<KHH, kAllLive, kExact>, cmap, wmap, qmap, a,
                               v_scales);
 }

@@ -492,20 +492,6 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
     const int ro = route_tiles;
     const uint32_t tmem_cols = route_pq ? kTmemColsPq : kTmemCols;
 
-    // Loads that do not depend on one another go out first, so their latency overlaps the
-    // set-up: the length, the append position and (producer) the split's first block-table
-    // entries, 32 pages per warp load, two batches.
-    const int L_raw = a.seq_lens[b];
-    const int pos_raw = a.v_new ? a.positions[b] : -1;
-    const int t_begin = split0 * geo.chunk;
-    const int first_page = t_begin / geo.P;
-    const int32_t *bt = a.block_table + (size_t)b * geo.max_pages;
-    int bt_cur = -1, bt_nxt = -1;
-    if (warp == kProducerWarp) {
-        if (first_page + lane < geo.max_pages) bt_cur = bt[first_page + lane];
-        if (first_page + 32 + lane < geo.max_pages) bt_nxt = bt[first_page + 32 + lane];
-    }
-
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
             ptx::mbar_init(&sm.full[s], 1);
@@ -548,6 +534,22 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
             ptx::prefetch_tensormap(&qmap);
         }
     }
+    // Nothing above touched global memory: past this point the kernels ahead in the stream have
+    // completed (the latent decode waits for the absorbed queries further down instead).
+    if (!a.pdl) grid_dep_wait();
+    // Loads that do not depend on one another go out at once: the length, the append position
+    // and (producer) the split's first block-table entries, 32 pages per warp load, two batches.
+    const int L_raw = a.seq_lens[b];
+    const int pos_raw = a.v_new ? a.positions[b] : -1;
+    const int t_begin = split0 * geo.chunk;
+    const int first_page = t_begin / geo.P;
+    const int32_t *bt = a.block_table + (size_t)b * geo.max_pages;
+    int bt_cur = -1, bt_nxt = -1;
+    if (warp == kProducerWarp) {
+        if (first_page + lane < geo.max_pages) bt_cur = bt[first_page + lane];
+        if (first_page + 32 + lane < geo.max_pages) bt_nxt = bt[first_page + 32 + lane];
+    }
+
     // Ring position r < route_tiles: W^R as the MN-major A operand [j half][128 k rows][128 B];
     // position 0 also brings the group's query rows as the K-major B operand (rows 0..G-1 of
     // the q_r buffer). Issued by the producer warp.
@@ -587,8 +589,7 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    // a kernel launched behind this one as a programmatic dependent (the combine of the split
-    // states, the latent expansion) may start setting up once every CTA is here
+    // the kernel behind this one may start setting up once every CTA is here
     grid_dep_launch();
     // The routing loads that fit the ring depend on nothing the CTA still reads (the length,
     // the block table), so they go out at once: the routed query is then ready about when
@@ -1321,13 +1322,7 @@ cudaError_t launch_kernel(const DecodeArgs &la, const CUtensorMap &vmap, const C
     cfg.blockDim = dim3(Roles<KH>::kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = la.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    if (la.pdl) {
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, decode_tc_kernel<kStandard, kPerSplit, KH, kExact, kD64>, vmap, kmap,
                               wmap, qmap, la);
 }

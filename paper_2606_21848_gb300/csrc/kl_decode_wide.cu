@@ -170,16 +170,6 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     const bool route_pq = route && geo.wr_per_qh;
     const int ro = !route ? 0 : route_pq ? G : 1;        // ring positions of W^R matrices
 
-    const int L_raw = a.seq_lens[b];
-    const int pos_raw = a.v_new ? a.positions[b] : -1;
-    const int t_begin = split0 * geo.chunk;
-    const int first_page = t_begin / geo.P;
-    const int32_t *bt = a.block_table + (size_t)b * geo.max_pages;
-    int bt_cur = -1, bt_nxt = -1;
-    if (warp == kWideProducer) {
-        if (first_page + lane < geo.max_pages) bt_cur = bt[first_page + lane];
-        if (first_page + 32 + lane < geo.max_pages) bt_nxt = bt[first_page + 32 + lane];
-    }
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) {
             ptx::mbar_init(&sm.full[s], 1);
@@ -213,6 +203,17 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             ptx::prefetch_tensormap(&qmap);
         }
     }
+    grid_dep_wait();        // nothing above touched global memory
+    const int L_raw = a.seq_lens[b];
+    const int pos_raw = a.v_new ? a.positions[b] : -1;
+    const int t_begin = split0 * geo.chunk;
+    const int first_page = t_begin / geo.P;
+    const int32_t *bt = a.block_table + (size_t)b * geo.max_pages;
+    int bt_cur = -1, bt_nxt = -1;
+    if (warp == kWideProducer) {
+        if (first_page + lane < geo.max_pages) bt_cur = bt[first_page + lane];
+        if (first_page + 32 + lane < geo.max_pages) bt_nxt = bt[first_page + 32 + lane];
+    }
     // Ring position r < ro: W^R as the MN-major A operand [j half][128 k rows][128 B]; position 0
     // also brings the CTA's query rows, the K-major B operand, into the front of the q_r buffer.
     auto issue_route = [&](int r) {
@@ -233,6 +234,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    grid_dep_launch();
     // the routing loads that fit the ring depend on nothing the CTA still reads
     const int early_route = ro < NS ? ro : NS;
     if (warp == kWideProducer)
@@ -757,6 +759,7 @@ cudaError_t launch_wide(const DecodeArgs &la, const CUtensorMap &vmap, const CUt
     cfg.blockDim = dim3(kWideThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = la.stream;
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, decode_wide_kernel<NH, kExact>, vmap, wmap, qmap, la);
 }
 

@@ -13,9 +13,11 @@ constexpr int kD = 128;
 // 4j .. 4j + 3. scale = max |v| / 448 (fp32), code = E4M3(v / scale) rounded to nearest even,
 // saturating.
 __global__ void __launch_bounds__(256)
-    append_fp8_kernel(int Hkv, int P, int num_pages, int max_pages, const uint16_t *__restrict__ v_new,
-                      const int32_t *__restrict__ block_table, const int32_t *__restrict__ positions,
-                      uint8_t *__restrict__ codes, float *__restrict__ scales, int32_t *err) {
+    append_fp8_kernel(int Hkv, int P, int num_pages, int max_pages, const uint16_t *v_new,
+                      const int32_t *block_table, const int32_t *positions,
+                      uint8_t *codes, float *scales, int32_t *err) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int b = blockIdx.x, lane = threadIdx.x & 31;
     const int pos = positions[b];
     if (pos < 0 || pos >= max_pages * P) {
@@ -72,9 +74,13 @@ cudaError_t launch_append_fp8(const Geometry &g, const uint16_t *v_new, const in
                               const int32_t *positions, uint8_t *codes, float *scales, int32_t *err,
                               cudaStream_t stream) {
     if (g.B == 0) return cudaSuccess;
-    append_fp8_kernel<<<g.B, 256, 0, stream>>>(g.Hkv, g.P, g.num_pages, g.max_pages, v_new,
-                                               block_table, positions, codes, scales, err);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g.B);
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    const OverlapAttr overlap(cfg);
+    return cudaLaunchKernelEx(&cfg, append_fp8_kernel, g.Hkv, g.P, g.num_pages, g.max_pages, v_new,
+                              block_table, positions, codes, scales, err);
 }
 
 cudaError_t launch_quantize_fp8(size_t rows, const uint16_t *v, uint8_t *codes, float *scales,

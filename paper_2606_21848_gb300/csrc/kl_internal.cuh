@@ -69,10 +69,10 @@ struct DecodeArgs {
     // Limit of each pipeline wait of the tensor-core decodes (ns); the drains of a CTA that gave
     // up keep the full default so that its copies and MMAs complete before it exits.
     uint64_t wait_ns = kDefaultWaitNs;
-    // Latent path: the launch is a programmatic dependent of the absorbed-query kernel ahead of
-    // it; the CTAs set up and fill their ring of cache tiles at once, every role then sleeps in
-    // grid_dep_wait until that kernel has finished (the compute warps before reading q_routed),
-    // and every CTA lets the expansion kernel behind it launch early (grid_dep_launch).
+    // Latent path, behind the absorbed-query kernel (which signals once everything ahead of it in
+    // the stream has completed): the CTAs set up and fill their ring of cache tiles at once,
+    // every role then sleeps in grid_dep_wait until that kernel has finished (the compute warps
+    // before reading q_routed).
     bool pdl = false;
 };
 
@@ -113,17 +113,34 @@ __device__ __forceinline__ void grid_dep_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Launch attribute of every kernel here: a programmatic dependent of the kernel ahead of it in the
+// stream. Where that kernel signals early (these kernels do, once all of their CTAs run), the
+// launch latency and the set-up overlap its end; each kernel calls grid_dep_wait() in all threads
+// before its first access to global memory (through pointers without __restrict__, whose loads
+// the compiler may not move above the wait), so stream order holds for everything it reads and
+// writes, and signals only once it holds its tensor memory, so that no CTA that waits for it can
+// take that. Behind any other kernel it starts as an ordinary launch. Calls one after another:
+// 8 x 4096 tokens 20.0 -> 16.9 us, one sequence of 131072 49.4 -> 47.0 us, 32 x 8192 at head dim
+// 64 86.2 -> 81.9 us, the 70B batch 604 -> 594 us.
+struct OverlapAttr {
+    cudaLaunchAttribute attr[1];
+    explicit OverlapAttr(cudaLaunchConfig_t &cfg) {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
+};
+
 // Launchers (each returns cudaGetLastError() of its launch).
 cudaError_t launch_append(const Geometry &g, const uint16_t *v_new, const int32_t *block_table,
                           const int32_t *positions, uint16_t *v_cache, int32_t *err,
                           cudaStream_t stream);
 cudaError_t launch_route(const Geometry &g, const uint16_t *q, const uint16_t *w_r, float *q_r,
                          cudaStream_t stream);
-// dependent: launched as a programmatic dependent of the decode just before it in the stream
-// (it starts once every decode CTA has set up and waits for the decode to complete)
 cudaError_t launch_combine(int B, int Hq, int D, int S, const float *part_o,
                            const float *part_ml, void *out, kl_dtype out_dtype,
-                           cudaStream_t stream, bool dependent = false);
+                           cudaStream_t stream);
 cudaError_t launch_decode_simt(const DecodeArgs &a, bool standard);
 // Merges the split states of a finished decode into `out` unless it wrote `out` directly or
 // the caller asked for the states.

@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nh = D / 64;                     // 64-value halves of a query row
     setup(sm, warp);
+    grid_dep_wait();
     const uint32_t tmem = sm.tmem_base;
     uint8_t *const q_s = sm.stage, *const wr_s = sm.stage + 2 * kBox;
 
@@ -496,6 +497,7 @@ cudaError_t launch_latent_query(int B, int Hq, int G, int D, int r, int wr_per_q
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, latent_query_kernel, qmap, wrmap, wpmap, qlmap, D, G, wr_per_qh,
                               err);
 }
@@ -520,12 +522,7 @@ cudaError_t launch_latent_expand(int B, int Hq, int D, int r, const float *o_lat
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmemBytes;
     cfg.stream = stream;
-    // a programmatic dependent of the decode (or of its combine kernel)
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, latent_expand_kernel, olmap, wpmap, outmap, D, (int)fp32, err);
 }
 

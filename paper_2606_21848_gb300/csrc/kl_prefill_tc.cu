@@ -215,6 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int mblk = (int)gridDim.z - 1 - (int)blockIdx.z;   // the longest blocks start first
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
+    grid_dep_wait();
     const int q0 = a.cu_q[b], q1 = a.cu_q[b + 1];
     const int L = a.seq_lens[b];
     const int n = q1 - q0;
@@ -268,6 +269,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    // the kernel behind may start setting up once every CTA is here (and holds its TMEM)
+    grid_dep_launch();
 
     const uint32_t tmem = sm.tmem_base;
     const Waiter wait{&sm.abort, a.err};
@@ -638,11 +641,13 @@ constexpr int kAppendRows = 16;
 
 __global__ void __launch_bounds__(128) append_chunk_kernel(int Hkv, int D, int P, int num_pages,
                                                            int max_pages, int total_q,
-                                                           const uint4 *__restrict__ v_new,
-                                                           const int32_t *__restrict__ block_table,
-                                                           const int32_t *__restrict__ seq_lens,
-                                                           const int32_t *__restrict__ cu_q,
-                                                           uint4 *__restrict__ v_cache, int32_t *err) {
+                                                           const uint4 *v_new,
+                                                           const int32_t *block_table,
+                                                           const int32_t *seq_lens,
+                                                           const int32_t *cu_q,
+                                                           uint4 *v_cache, int32_t *err) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int b = blockIdx.y;
     const int q0 = cu_q[b], n = cu_q[b + 1] - q0, L = seq_lens[b];
     if (q0 < 0 || n < 0 || q0 + n > total_q || L < n || L > max_pages * P) {
@@ -746,6 +751,7 @@ cudaError_t launch_prefill_tc(const PrefillArgs &a) {
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = a.stream;
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, prefill_tc_kernel, vmap, wmap, qmap, a);
 }
 
@@ -754,11 +760,14 @@ cudaError_t launch_append_chunk(const Geometry &g, int total_q, int max_q, const
                                 const int32_t *cu_q, uint16_t *v_cache, int32_t *err,
                                 cudaStream_t stream) {
     if (g.B == 0 || total_q == 0 || max_q == 0) return cudaSuccess;
-    const dim3 grid((max_q + kAppendRows - 1) / kAppendRows, g.B);
-    append_chunk_kernel<<<grid, 128, 0, stream>>>(g.Hkv, g.D, g.P, g.num_pages, g.max_pages, total_q,
-                                                  reinterpret_cast<const uint4 *>(v_new), block_table,
-                                                  seq_lens, cu_q, reinterpret_cast<uint4 *>(v_cache), err);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((max_q + kAppendRows - 1) / kAppendRows, g.B);
+    cfg.blockDim = dim3(128);
+    cfg.stream = stream;
+    const OverlapAttr overlap(cfg);
+    return cudaLaunchKernelEx(&cfg, append_chunk_kernel, g.Hkv, g.D, g.P, g.num_pages, g.max_pages,
+                              total_q, reinterpret_cast<const uint4 *>(v_new), block_table, seq_lens,
+                              cu_q, reinterpret_cast<uint4 *>(v_cache), err);
 }
 
 }  // namespace kl

@@ -9,10 +9,12 @@ namespace {
 // Append (Section 3): one CTA per sequence copies the Hkv value rows of the current token
 // into row pos % P of page block_table[b][pos / P]. 16-byte copies; D is a multiple of 8.
 __global__ void __launch_bounds__(128) append_kernel(int Hkv, int D, int P, int num_pages,
-                                                     int max_pages, const uint4 *__restrict__ v_new,
-                                                     const int32_t *__restrict__ block_table,
-                                                     const int32_t *__restrict__ positions,
-                                                     uint4 *__restrict__ v_cache, int32_t *err) {
+                                                     int max_pages, const uint4 *v_new,
+                                                     const int32_t *block_table,
+                                                     const int32_t *positions,
+                                                     uint4 *v_cache, int32_t *err) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int b = blockIdx.x;
     const int pos = positions[b];
     if (pos < 0 || pos >= max_pages * P) {
@@ -57,8 +59,8 @@ constexpr int kCombineWarps = 4;
 constexpr int kCombineMaxSplits = 1024;
 
 __global__ void __launch_bounds__(kCombineWarps * 32)
-    combine_kernel(int Hq, int D, int S, const float *__restrict__ part_o,
-                   const float2 *__restrict__ part_ml, void *out, int out_fp32) {
+    combine_kernel(int Hq, int D, int S, const float *part_o,
+                   const float2 *part_ml, void *out, int out_fp32) {
     __shared__ float w_s[kCombineMaxSplits];
     __shared__ float red[kCombineWarps];
     __shared__ float4 acc_s[kCombineWarps][32];
@@ -66,9 +68,8 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t bh = (size_t)b * Hq + h;
     const float2 *ml = part_ml + bh * S;
-    // behind a decode as its programmatic dependent: the decode's states are complete and
-    // visible past this point (an ordinary launch returns at once)
-    grid_dep_wait();
+    grid_dep_wait();      // the states are complete and visible past this point
+    grid_dep_launch();
 
     float M = -INFINITY;
     for (int s = tid; s < S; s += blockDim.x) {
@@ -132,10 +133,14 @@ cudaError_t launch_append(const Geometry &g, const uint16_t *v_new, const int32_
                           const int32_t *positions, uint16_t *v_cache, int32_t *err,
                           cudaStream_t stream) {
     if (g.B == 0) return cudaSuccess;
-    append_kernel<<<g.B, 128, 0, stream>>>(g.Hkv, g.D, g.P, g.num_pages, g.max_pages,
-                                           reinterpret_cast<const uint4 *>(v_new), block_table,
-                                           positions, reinterpret_cast<uint4 *>(v_cache), err);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(g.B);
+    cfg.blockDim = dim3(128);
+    cfg.stream = stream;
+    const OverlapAttr overlap(cfg);
+    return cudaLaunchKernelEx(&cfg, append_kernel, g.Hkv, g.D, g.P, g.num_pages, g.max_pages,
+                              reinterpret_cast<const uint4 *>(v_new), block_table, positions,
+                              reinterpret_cast<uint4 *>(v_cache), err);
 }
 
 cudaError_t launch_route(const Geometry &g, const uint16_t *q, const uint16_t *w_r, float *q_r,
@@ -147,20 +152,14 @@ cudaError_t launch_route(const Geometry &g, const uint16_t *q, const uint16_t *w
 
 cudaError_t launch_combine(int B, int Hq, int D, int S, const float *part_o,
                            const float *part_ml, void *out, kl_dtype out_dtype,
-                           cudaStream_t stream, bool dependent) {
+                           cudaStream_t stream) {
     if (B == 0) return cudaSuccess;
     if (S > kCombineMaxSplits) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(Hq, B);
     cfg.blockDim = dim3(kCombineWarps * 32);
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    if (dependent) {
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
+    const OverlapAttr overlap(cfg);
     return cudaLaunchKernelEx(&cfg, combine_kernel, Hq, D, S, part_o,
                               reinterpret_cast<const float2 *>(part_ml), out,
                               (int)(out_dtype == KL_FP32));
