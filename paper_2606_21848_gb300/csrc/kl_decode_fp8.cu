@@ -10,13 +10,23 @@
 //   scores   S^T = C_t . Q^T     M = 128 tokens, N = 32, K = 128 dims    (C_t K-major)
 //   output   O^T = C_t^T . W     M = 128 dims,   N = 32, K = 128 tokens  (C_t MN-major)
 //
+// (N = 16 for CTAs of up to 4 heads.)
+//
 // The other operands keep more precision than one E4M3 value by being sums of E4M3 terms in
 // separate columns: each term is the rounding residual of the previous one times 16, so each
 // adds four significant bits. Q holds the routed query (times scale * log2 e) of the 8 heads as
-// 4 terms, W the softmax weights times the row scales as 3 terms; head h = 4 hh + k, term j sits
-// in score column 16 hh + 4 j + k and output column 16 hh + 4 j + k (output columns 12..15 of
-// each half zero). Before the split a power of two brings the operand's largest value below
+// 4 terms, W the softmax weights times the row scales as 3 terms; head h = 4 blk + k, term j sits
+// in score column 16 blk + 4 j + k and output column 16 blk + 4 j + k (output columns 12..15 of
+// each block zero). Before the split a power of two brings the operand's largest value below
 // 256 (E4M3 reaches 448); it is divided out again after the terms are summed.
+//
+// The compute warps' instructions set the pace here (each token carries half the bytes of a bf16
+// row and more arithmetic), and most of them were per warp and tile, not per head: waits, votes,
+// addresses. So the eight compute warps form two groups of four that take alternate tiles, each
+// thread with all (8 or 4) heads of its token, and each group with its own softmax state and O,
+// merged at the end like two splits. With all eight warps on every tile, half the heads each, the
+// 70B batch (256 x 64/8 heads, 8192 tokens) ran 437 us, now 370 us (the HBM floor is 327);
+// 64 ragged sequences of 32/8 heads 254 -> 204 us, together with the one-lane page loop.
 //
 // The softmax keeps a lazy reference maximum per head: a tile's weights are 2^(s - m) with the
 // current reference m, and m moves (rescaling the running sums) only when a score passes it by
@@ -28,11 +38,10 @@
 // (p_t scale_t), so the codes are used as stored.
 //
 // One CTA per (split, value head g, sequence b); 352 threads, two CTAs per SM:
-//   warps 0-7  compute. Warp w reads TMEM lane quarter w % 4 and takes heads 4 (w / 4) .. + 3:
-//              routing result and query split (thread = dim); per tile the online softmax in
-//              base 2 and the weight split (thread = token), O accumulation (thread = output
-//              dim); epilogue (output row or split state). Two warps per lane quarter halve
-//              the per-thread work of a tile, which bounds the tile rate.
+//   warps 0-7  compute. Warp w reads TMEM lane quarter w % 4 and belongs to group w / 4:
+//              routing result and query split (thread = dim); per tile of the group the online
+//              softmax in base 2 and the weight split (thread = token); epilogue (thread =
+//              output dim: output row or split state)
 //   warp 8     producer: W^R[g] (ring stages 0-1) and the group's query rows, then per tile the
 //              TMA loads of code pages and bulk copies of their scale rows; for the decode step
 //              (kl_decode_step_fp8) it first quantizes the current token's row into the cache
@@ -57,9 +66,9 @@ constexpr int kTile = 128;
 constexpr int kJq = 4;                      // E4M3 terms of the routed query
 constexpr int kJp = 3;                      // E4M3 terms of the weights
 constexpr int kNR = 16;                     // routing MMA N (query rows, padded)
-constexpr int kQuarters = 4;                // TMEM lane quarters (warps per head half)
-constexpr int kComputeWarps = 8;
+constexpr int kComputeWarps = 8;            // two groups of four
 constexpr int kComputeThreads = kComputeWarps * 32;
+constexpr int kGroupThreads = 128;
 constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
 constexpr int kPvWarp = 10;
@@ -68,28 +77,26 @@ constexpr int kStages = 5;
 constexpr uint32_t kCodeBytes = kTile * kD;          // 16 KiB of codes per tile
 constexpr uint32_t kHalfBytes = 16384;               // one 64-column half of W^R (bf16)
 constexpr uint32_t kPBytes = 4096;                   // weight operand buffer (largest shape)
-constexpr int kPBuf = 4;                             // weight operands in flight
-constexpr uint32_t kTmemCols = 128;
+constexpr int kBuf = 4;                              // score and weight buffers, two per group
+constexpr uint32_t kTmemCols = 256;
 constexpr uint32_t kColS = 0;                        // S[b]: columns 32 b .. 32 b + 31
-constexpr uint32_t kColO = 64;                       // O: columns 64 .. 95, summed over tiles
-constexpr uint32_t kColR = 96;                       // routing result: 96 .. 111
+constexpr uint32_t kColO = 128;                      // O of group i: 128 + 32 i .., summed over
+                                                     // the group's tiles
+constexpr uint32_t kColR = 192;                      // routing result: 192 .. 207
 constexpr float kLazyW = 4.f;                        // reference slack: weights 2^(s - m) <= 4
 constexpr uint64_t kTimeoutNs = kDefaultWaitNs;   // bound of the drains
 constexpr uint32_t kSleepHintNs = 20000u;         // suspend hint of a wait that did not finish at once
-constexpr uint32_t kBarCompute = 1;
 constexpr uint32_t kBarComputeAnd = 2;
+constexpr uint32_t kBarGroup = 3;                 // + group
 
-// Operand shapes for KHH query heads per compute warp (4 when the group has 5..8 heads, 2 when
-// it has at most 4, so that no compute warp carries only padded heads). Head h = KHH hh + k
-// (hh = warp / 4) and term j sit in score column HS hh + KHH j + k and output column
-// HP hh + KHH j + k.
-template <int KHH>
+// Operand shapes for NB blocks of 4 query heads (2 when the CTA has 5..8 heads, 1 when it has at
+// most 4). Head h = 4 blk + k and term j sit in score column 16 blk + 4 j + k and output column
+// 16 blk + 4 j + k.
+template <int NB>
 struct Fp8Shape {
-    static constexpr int NS = 8 * KHH;        // score MMA N: 4 query terms x 2 KHH heads
-    static constexpr int NP = 8 * KHH;        // output MMA N: 3 weight terms x 2 KHH heads, padded
-    static constexpr int HS = NS / 2;         // score columns of one warp
-    static constexpr int HP = NP / 2;         // output columns of one warp
-    static constexpr int GS = 8 * NP;         // weight operand: bytes per group of 8 tokens
+    static constexpr int NH = 4 * NB;         // query heads (padded)
+    static constexpr int N = 16 * NB;         // MMA N: 4 query terms, or 3 weight terms padded
+    static constexpr int GS = 8 * N;          // weight operand: bytes per group of 8 tokens
 };
 
 struct __align__(1024) Smem8 {
@@ -98,14 +105,18 @@ struct __align__(1024) Smem8 {
     uint8_t codes[kStages][kCodeBytes];
     // Query terms, B operand of the score MMAs: [NS rows n][128 dims], K-major, 128B-swizzled.
     uint8_t qt[32 * 128];
-    // Weight terms, B operand of the output MMAs: [16 groups of 8 tokens][NP / 16 blocks of 16
+    // Weight terms, B operand of the output MMAs: [16 groups of 8 tokens][N / 16 blocks of 16
     // columns][8 tokens][16 B], MN-major, no swizzle. During the routing prologue the first one
     // holds the query rows: [64-dim half][16 rows][128 B], K-major, 128B-swizzled.
-    uint8_t p[kPBuf][kPBytes];
+    uint8_t p[kBuf][kPBytes];
     float scl[kStages][kTile];         // row scales of each stage's tile, token order
-    float red[2][kComputeWarps][8];    // per warp: 4 head maxima (or row sums), the scale max
+    float red[2][4][12];               // per group and lane quarter: 8 head maxima (or row sums),
+                                       // then the scale maximum
+    float mref[2][8];                  // per group: the heads' references
+    float invq[8];                     // per head: the inverse power of its query terms
+    float winv[2];                     // per group: the inverse power of its weights
     uint64_t full[kStages], empty[kStages];
-    uint64_t s_full[2], s_empty[2], p_full[kPBuf], o_full[kPBuf];
+    uint64_t s_full[kBuf], s_empty[kBuf], p_full[kBuf], o_full[kBuf];
     uint64_t r_full, qt_full, drain, drain2;
     uint32_t tmem_base;
     int abort;
@@ -260,62 +271,14 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&u)[16
         : "memory");
 }
 
-// 8 consecutive 32-bit columns of the thread's TMEM lane (load and wait in one statement).
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8]) {
-    uint32_t u[8];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
-          "=r"(u[7])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 8; ++i) r[i] = __uint_as_float(u[i]);
-}
-
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&u)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(
-                     taddr),
-                 "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]), "r"(u[4]), "r"(u[5]), "r"(u[6]),
-                 "r"(u[7])
-                 : "memory");
-}
-
-// N (8 or 16) consecutive columns of the thread's TMEM lane.
-template <int N>
-__device__ __forceinline__ void tmem_ldn(uint32_t taddr, float (&r)[N]) {
-    if constexpr (N == 16) ptx::tmem_ld16(taddr, r);
-    else tmem_ld8(taddr, r);
-}
-template <int N>
-__device__ __forceinline__ void tmem_stn(uint32_t taddr, const uint32_t (&u)[N]) {
-    if constexpr (N == 16) tmem_st16(taddr, u);
-    else tmem_st8(taddr, u);
-}
-
-// Barrier `id` over `count` threads that also returns how many of them passed v = true.
-__device__ __forceinline__ uint32_t bar_popc(uint32_t id, uint32_t count, bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.popc.u32 %0, %2, %3, p;\n\t}\n"
-        : "=r"(r)
-        : "r"((uint32_t)v), "r"(id), "r"(count)
-        : "memory");
-    return r;
-}
-
-template <int KHH, bool kAllLive, bool kExact>
+template <int NB, bool kExact>
 __global__ void __launch_bounds__(kThreads, 2)
     decode_fp8_kernel(const __grid_constant__ CUtensorMap cmap,
                       const __grid_constant__ CUtensorMap wmap,
                       const __grid_constant__ CUtensorMap qmap, const DecodeArgs a,
                       const float *v_scales) {
-    using Sh = Fp8Shape<KHH>;
+    using Sh = Fp8Shape<NB>;
     extern __shared__ uint8_t smem_raw[];
-    // kAllLive: the group has 2 KHH heads, so no compute warp holds a padded head
     Smem8 &sm = *reinterpret_cast<Smem8 *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                            ~uintptr_t(1023));
     const Geometry &geo = a.geo;
@@ -336,12 +299,10 @@ __global__ void __launch_bounds__(kThreads, 2)
             ptx::mbar_init(&sm.full[s], 1);
             ptx::mbar_init(&sm.empty[s], 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < kBuf; ++i) {
             ptx::mbar_init(&sm.s_full[i], 1);
-            ptx::mbar_init(&sm.s_empty[i], kComputeWarps);
-        }
-        for (int i = 0; i < kPBuf; ++i) {
-            ptx::mbar_init(&sm.p_full[i], kComputeWarps);
+            ptx::mbar_init(&sm.s_empty[i], kComputeWarps / 2);
+            ptx::mbar_init(&sm.p_full[i], kComputeWarps / 2);
             ptx::mbar_init(&sm.o_full[i], 1);
         }
         ptx::mbar_init(&sm.r_full, 1);
@@ -351,6 +312,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         sm.abort = 0;
         ptx::fence_mbar_init();
     }
+    if (tid < 16) (&sm.mref[0][0])[tid] = -INFINITY;
     if (warp == kMmaWarp) {
         ptx::tmem_alloc(&sm.tmem_base, kTmemCols);
         ptx::tmem_relinquish();
@@ -482,14 +444,14 @@ __global__ void __launch_bounds__(kThreads, 2)
             const bool in_range = exists && page >= 0 && page < geo.num_pages;
             if (exists && !in_range) bad = true;
             const unsigned mask = __ballot_sync(0xffffffffu, in_range);
-            if (lane == 0) ptx::mbar_arrive_expect_tx(&sm.full[s], __popc(mask) * page_bytes);
-            __syncwarp();
-            if (in_range) {
-                const int row = (page * geo.Hkv + g) * P;
-                ptx::tma_load_2d(sm.codes[s] + lane * P * 128, &cmap, &sm.full[s], 0, row);
-                ptx::bulk_load(&sm.scl[s][lane * P], v_scales + (size_t)row, (uint32_t)P * 4u,
-                               &sm.full[s]);
-            }
+            ptx::for_pages(
+                (page * geo.Hkv + g) * P, mask,
+                [&] { ptx::mbar_arrive_expect_tx(&sm.full[s], __popc(mask) * page_bytes); },
+                [&](int p, int row) {
+                    ptx::tma_load_2d(sm.codes[s] + p * P * 128, &cmap, &sm.full[s], 0, row);
+                    ptx::bulk_load(&sm.scl[s][p * P], v_scales + (size_t)row, (uint32_t)P * 4u,
+                                   &sm.full[s]);
+                });
             issued = u + 1;
         }
         if (__any_sync(0xffffffffu, bad) && lane == 0) raise_flag(a.err, KL_FLAG_BAD_PAGE);
@@ -524,14 +486,14 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         ok = ok && wait(&sm.qt_full, 0);
         if (ok) ptx::tc_fence_after();
-        constexpr uint32_t idesc_s = idesc_f8(128, Sh::NS, false, false);
+        constexpr uint32_t idesc_s = idesc_f8(128, Sh::N, false, false);
         const uint64_t c_desc =
             ptx::smem_desc(ptx::smem_addr(sm.codes[0]), 16, 1024, ptx::kSwizzle128B);
         const uint64_t q_desc = ptx::smem_desc(ptx::smem_addr(sm.qt), 16, 1024, ptx::kSwizzle128B);
         for (int i = 0; ok && i < n_tiles; ++i) {
-            const int u = i + base, s = u % kStages, sb = i & 1;
+            const int u = i + base, s = u % kStages, sb = i % kBuf;
             if (!wait(&sm.full[s], (u / kStages) & 1)) break;
-            if (i >= 2 && !wait(&sm.s_empty[sb], ((i >> 1) - 1) & 1)) break;
+            if (i >= kBuf && !wait(&sm.s_empty[sb], (i / kBuf - 1) & 1)) break;
             ptx::tc_fence_after();
             if (ptx::elect_one()) {
                 const uint64_t a0 = c_desc + ((s * kCodeBytes) >> 4);
@@ -552,14 +514,14 @@ __global__ void __launch_bounds__(kThreads, 2)
         // ------------------------------------------------------ output MMA issuer -------
         // A = C^T: the code tile read MN-major (8-token row groups 1 KiB apart); B = W:
         // MN-major, no swizzle (16-column blocks 128 B apart, 8-token groups GS bytes apart)
-        constexpr uint32_t idesc_o = idesc_f8(128, Sh::NP, true, true);
+        constexpr uint32_t idesc_o = idesc_f8(128, Sh::N, true, true);
         const uint64_t c_desc =
             ptx::smem_desc(ptx::smem_addr(sm.codes[0]), 8192, 1024, ptx::kSwizzle128B);
         const uint64_t p_desc =
             ptx::smem_desc(ptx::smem_addr(sm.p[0]), Sh::GS, 128, ptx::kSwizzleNone);
         for (int j = 0; j < n_tiles; ++j) {
-            const int u = j + base, s = u % kStages, pb = j % kPBuf;
-            if (!wait(&sm.p_full[pb], (j / kPBuf) & 1)) break;
+            const int u = j + base, s = u % kStages, pb = j % kBuf;
+            if (!wait(&sm.p_full[pb], (j / kBuf) & 1)) break;
             ptx::tc_fence_after();
             const int nvalid = min(kTile, t_end - (t_begin + j * kTile));
             const int ksteps = (nvalid + 31) >> 5;
@@ -567,9 +529,9 @@ __global__ void __launch_bounds__(kThreads, 2)
                 const uint64_t a0 = c_desc + ((s * kCodeBytes) >> 4);
                 const uint64_t b0 = p_desc + ((pb * kPBytes) >> 4);
                 for (int kk = 0; kk < ksteps; ++kk)
-                    mma_f8(tmem + kColO, a0 + ((kk * 4096) >> 4), b0 + ((kk * 4 * Sh::GS) >> 4),
-                           idesc_o, (j > 0 || kk > 0) ? 1u : 0u);
-                ptx::mma_commit(&sm.o_full[pb]);   // tile j: phase j / kPBuf of o_full[j % kPBuf]
+                    mma_f8(tmem + kColO + (j & 1) * 32, a0 + ((kk * 4096) >> 4),
+                           b0 + ((kk * 4 * Sh::GS) >> 4), idesc_o, (j > 1 || kk > 0) ? 1u : 0u);
+                ptx::mma_commit(&sm.o_full[pb]);   // tile j: phase j / kBuf of o_full[j % kBuf]
                 ptx::mma_commit(&sm.empty[s]);     // the tile's last reader is done
             }
             __syncwarp();
@@ -581,66 +543,57 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
     } else {
         // ------------------------------------------------------------------ compute -----
-        // Warp w: TMEM lane quarter q4 = w % 4 (dims / tokens 32 q4 .. 32 q4 + 31) and heads
-        // h = 4 hh + k (k = 0..3) with hh = w / 4.
-        const int q4 = warp & 3, hh = warp >> 2;
+        // Warp w: TMEM lane quarter q4 = w % 4 (dims / tokens 32 q4 .. 32 q4 + 31), group w / 4.
+        const int q4 = warp & 3, grp = warp >> 2;
         const int t = q4 * 32 + lane;                       // dim / token / output dim
         const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
-        const float sl2 = geo.scale * kLog2e;
         bool ok = true;
 
-        // Routed query: from the routing MMA (TMEM), or the composed query itself.
-        float acc[KHH];
+        // Prologue and epilogue: the groups share the heads, h1 .. h1 + KR - 1 each.
+        constexpr int KR = 2 * NB;
+        const int h1 = KR * grp;
+        // Routed query (thread = dim t) from the routing MMA (TMEM), or the composed query itself.
+        float acc[KR];
 #pragma unroll
-        for (int k = 0; k < KHH; ++k) acc[k] = 0.f;
+        for (int e = 0; e < KR; ++e) acc[e] = 0.f;
         if (route) {
-            ok = ptx::bar_and(kBarComputeAnd, kComputeThreads, wait(&sm.r_full, 0));
+            ok = ptx::bar_and(kBarGroup + grp, kGroupThreads, wait(&sm.r_full, 0));
             if (ok) {
                 ptx::tc_fence_after();
-                float rv[16];
-                ptx::tmem_ld16(tmem + kColR + lane_base, rv);
 #pragma unroll
-                for (int k = 0; k < KHH; ++k)
-                    acc[k] = (kAllLive || KHH * hh + k < G) ? (hh ? rv[KHH + k] : rv[k]) : 0.f;
+                for (int e = 0; e < KR; ++e)
+                    if (h1 + e < G) acc[e] = ptx::tmem_ld1(tmem + kColR + h1 + e + lane_base);
                 ptx::tc_fence_before();
             }
         } else {
 #pragma unroll
-            for (int k = 0; k < KHH; ++k) {
-                const int h = KHH * hh + k;
-                acc[k] = h < G ? __uint_as_float((uint32_t)a.q[((size_t)b * geo.Hq + qh0 + h) * kD + t] << 16)
-                               : 0.f;
-            }
+            for (int e = 0; e < KR; ++e)
+                if (h1 + e < G)
+                    acc[e] = __uint_as_float((uint32_t)a.q[((size_t)b * geo.Hq + qh0 + h1 + e) * kD + t] << 16);
         }
-        // Query terms: per head, 2^(8 - e) over its largest |value|, then 6 E4M3 terms.
-        float invq[KHH];
+        // Query terms: per head, 2^(8 - e) over its largest |value|, then 4 E4M3 terms. A padded
+        // head has zero terms: its scores are 0, finite, and it is never written out.
         if (ok) {
-            float v[KHH], av[KHH];
+            const float sl2 = geo.scale * kLog2e;
 #pragma unroll
-            for (int k = 0; k < KHH; ++k) {
-                v[k] = acc[k] * sl2;
-                av[k] = fabsf(v[k]);
+            for (int e = 0; e < KR; ++e) {
+                acc[e] *= sl2;
+                const float wm = warp_max(fabsf(acc[e]));
+                if (lane == 0) sm.red[grp][q4][e] = wm;
             }
-            float wm[KHH];
+            ptx::bar_sync(kBarGroup + grp, kGroupThreads);
 #pragma unroll
-            for (int k = 0; k < KHH; ++k) wm[k] = warp_max(av[k]);
-            if (lane == 0) {
-#pragma unroll
-                for (int k = 0; k < KHH; ++k) sm.red[1][warp][k] = wm[k];
-            }
-            ptx::bar_sync(kBarCompute, kComputeThreads);
-#pragma unroll
-            for (int k = 0; k < KHH; ++k) {
-                float amax = sm.red[1][kQuarters * hh][k];
-#pragma unroll
-                for (int w = 1; w < 4; ++w) amax = fmaxf(amax, sm.red[1][kQuarters * hh + w][k]);
-                float sc;
-                pow2_scale(amax, sc, invq[k]);
-                float x = v[k] * sc;
+            for (int e = 0; e < KR; ++e) {
+                const float amax = fmaxf(fmaxf(sm.red[grp][0][e], sm.red[grp][1][e]),
+                                         fmaxf(sm.red[grp][2][e], sm.red[grp][3][e]));
+                float sc, inv;
+                pow2_scale(amax, sc, inv);
+                if (t == 0) sm.invq[h1 + e] = inv;
+                float x = acc[e] * sc;
 #pragma unroll
                 for (int j = 0; j < kJq; ++j) {
                     const __nv_fp8_storage_t c = __nv_cvt_float_to_fp8(x, __NV_SATFINITE, __NV_E4M3);
-                    sm.qt[qt_offset(Sh::HS * hh + KHH * j + k, t)] = c;
+                    sm.qt[qt_offset(16 * ((h1 + e) >> 2) + 4 * j + ((h1 + e) & 3), t)] = c;
                     x = (x - e4m3x2_to_float2((uint32_t)c).x) * 16.f;
                 }
             }
@@ -648,252 +601,243 @@ __global__ void __launch_bounds__(kThreads, 2)
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&sm.qt_full);
         }
+        // (both groups' invq before the first tile)
+        ok = ptx::bar_and(kBarComputeAnd, kComputeThreads, ok);
 
-        // m: the reference maximum of each head (0 for padded heads, whose scores are -inf);
-        // a weight 2^(s - m) past kLazyW moves it
-        float m[KHH], lsum[KHH];
+        // The group's softmax state: the references in shared memory (a weight 2^(s - m) past
+        // kLazyW moves them), this thread's share of the row sums.
+        float *const mref = sm.mref[grp];
+        float lsum[Sh::NH];
 #pragma unroll
-        for (int k = 0; k < KHH; ++k) {
-            const bool live = kAllLive || KHH * hh + k < G;
-            m[k] = live ? -INFINITY : 0.f;
-            lsum[k] = 0.f;
-        }
+        for (int h = 0; h < Sh::NH; ++h) lsum[h] = 0.f;
         // Lazy weight scale: every row scale so far is below lim = 2^es; weights are taken
-        // times sc = 2^(6 - es) and O times inv = 2^(es - 6) at the end.
+        // times sc = 2^(6 - es) and O times 2^(es - 6) at the end.
         int es = -1000;
         float lim = 0.f, sc = 1.f, inv = 1.f;
-        // Completions of the output MMAs: tile j is phase j / kPBuf of o_full[j % kPBuf]. The
-        // tiles are observed in order, and a warp observes tile i - kPBuf (the last reader of
-        // the weight buffer it is about to fill) before it releases tile i, so no barrier runs
-        // more than one phase ahead of its observer and no phase is mistaken for a later one of
-        // the same parity.
-        int o_seen = 0;                                // tiles 0 .. o_seen - 1 observed
-        auto observe = [&](int j) -> bool {            // the output MMAs up to tile j are done
-            while (o_seen <= j) {
-                if (!wait(&sm.o_full[o_seen % kPBuf], (o_seen / kPBuf) & 1)) return false;
-                ++o_seen;
-            }
-            return true;
-        };
-
-        // One barrier per tile for all compute warps: it counts the warps with a score past its
-        // reference, a row scale past lim, or a failed wait since the last barrier. Only then a
-        // second one exchanges the tile maxima (or lets all of them leave the loop together
-        // after a failed wait).
+        // One barrier of the group per tile: it counts the threads with a score past its
+        // reference, a row scale past lim, or a failed wait. Only then a second one exchanges
+        // the tile maxima (or lets the group leave together after a failed wait).
         bool carried = true;
-        for (int i = 0; ok && i < n_tiles; ++i) {
-            const int u = i + base, s = u % kStages, sb = i & 1;
-            // the stage's loads have landed (its scale row is read below), S is ready, and the
-            // output MMAs of tile i - kPBuf (the last reader of this weight buffer) are done
-            const int pb = i % kPBuf;
-            bool ready = wait(&sm.full[s], (u / kStages) & 1);
-            ready = ready && wait(&sm.s_full[sb], (i >> 1) & 1);
-            ready = ready && observe(i - kPBuf);
-            float sv[Sh::HS];
+        int st_i = (grp + base) % kStages, st_ph = 0;    // ring stage and phase of tile i
+        for (int i = grp; ok && i < n_tiles; i += 2) {
+            const int sb = i % kBuf;
+            const int nvalid = min(kTile, t_end - (t_begin + i * kTile));
+            const bool past = t >= nvalid;
+            const uint32_t scol = tmem + kColS + sb * 32 + lane_base;
+            // S is ready, so the tile has landed: then its stage's barrier, whose phase is that of
+            // this tile until its output MMAs are done, also orders the read of its scale row
+            bool ready = carried && wait(&sm.s_full[sb], (i / kBuf) & 1);
+            ready = ready && wait(&sm.full[st_i], st_ph);
+            // the row scale of token t (stale bytes past the end)
+            const float st = past ? 0.f : sm.scl[st_i][t];
+            float p_k[Sh::NH];
+            float pmax = 0.f;
+            // scores of block blk: the term columns 16^-j D_j summed from the last term (two
+            // heads at once), times the head's inverse power and the row scale
+            auto scores = [&](int blk, F2 &s01, F2 &s23) {
+                float sv[16];
+                ptx::tmem_ld16(scol + 16 * blk, sv);
+                const float4 iq = *reinterpret_cast<const float4 *>(&sm.invq[4 * blk]);
+                const F2 s16 = f2(1.f / 16.f, 1.f / 16.f), stt = f2(st, st);
+                s01 = mul2(fma2(fma2(fma2(f2(sv[12], sv[13]), s16, f2(sv[8], sv[9])), s16, f2(sv[4], sv[5])),
+                                s16, f2(sv[0], sv[1])),
+                           mul2(f2(iq.x, iq.y), stt));
+                s23 = mul2(fma2(fma2(fma2(f2(sv[14], sv[15]), s16, f2(sv[10], sv[11])), s16, f2(sv[6], sv[7])),
+                                s16, f2(sv[2], sv[3])),
+                           mul2(f2(iq.z, iq.w), stt));
+            };
             if (ready) {
                 ptx::tc_fence_after();
-                tmem_ldn<Sh::HS>(tmem + kColS + sb * 32 + Sh::HS * hh + lane_base, sv);
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&sm.s_empty[sb]);
-            } else {
 #pragma unroll
-                for (int c = 0; c < Sh::HS; ++c) sv[c] = 0.f;
-            }
-
-            const int nvalid = min(kTile, t_end - (t_begin + i * kTile));
-            const bool valid = t < nvalid;
-            float st = sm.scl[s][t];                      // the row scale of token t
-            if (nvalid < kTile && !valid) st = 0.f;       // (stale bytes past the end)
-            float s_k[KHH];
-#pragma unroll
-            for (int k = 0; k < KHH; k += 2) {
-                // sum of the term columns, 16^-j D_j, from the last term (two heads at once)
-                const F2 s16 = f2(1.f / 16.f, 1.f / 16.f);
-                const F2 d = fma2(fma2(fma2(f2(sv[3 * KHH + k], sv[3 * KHH + k + 1]), s16,
-                                            f2(sv[2 * KHH + k], sv[2 * KHH + k + 1])),
-                                       s16, f2(sv[KHH + k], sv[KHH + k + 1])),
-                                  s16, f2(sv[k], sv[k + 1]));
-                const F2 sk = mul2(d, mul2(f2(invq[k], invq[k + 1]), f2(st, st)));
-                s_k[k] = (kAllLive || KHH * hh + k < G) ? sk.x : -INFINITY;
-                s_k[k + 1] = (kAllLive || KHH * hh + k + 1 < G) ? sk.y : -INFINITY;
-            }
-            if (nvalid < kTile && !valid) {
-#pragma unroll
-                for (int k = 0; k < KHH; ++k) s_k[k] = -INFINITY;
-            }
-            // the weights against the current references; a weight past kLazyW moves them
-            float p_k[KHH];
-#pragma unroll
-            for (int k = 0; k < KHH; k += 2) {   // 0 for padded heads
-                const F2 e = sub2(f2(s_k[k], s_k[k + 1]), f2(m[k], m[k + 1]));
-                p_k[k] = ptx::ex2(e.x);
-                p_k[k + 1] = ptx::ex2(e.y);
-            }
-            float pmax = p_k[0];
-#pragma unroll
-            for (int k = 1; k < KHH; ++k) pmax = fmaxf(pmax, p_k[k]);
-            bool grow = pmax > kLazyW;
-            // row scales are non-negative: their bits order as the values do
-            const float smx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(st)));
-            grow = grow || smx >= lim;
-            if (lane == 0) sm.red[sb][warp][KHH] = smx;
-            const bool fine = ready && carried;
-            float alpha[KHH];
-#pragma unroll
-            for (int k = 0; k < KHH; ++k) alpha[k] = 1.f;
-            if (bar_popc(kBarComputeAnd, kComputeThreads, grow || !fine) != 0) {
-                // move the references to the heads' running maxima and lim past the row scales
-                float wm[KHH];
-#pragma unroll
-                for (int k = 0; k < KHH; ++k) wm[k] = warp_max(s_k[k]);
-                if (lane == 0) {
-#pragma unroll
-                    for (int k = 0; k < KHH; ++k) sm.red[sb][warp][k] = wm[k];
+                for (int blk = 0; blk < NB; ++blk) {
+                    F2 s01, s23;
+                    scores(blk, s01, s23);
+                    // the weights against the current references (0 past the end)
+                    const float4 m = *reinterpret_cast<const float4 *>(&mref[4 * blk]);
+                    s01 = sub2(s01, f2(m.x, m.y));
+                    s23 = sub2(s23, f2(m.z, m.w));
+                    float *p = p_k + 4 * blk;
+                    p[0] = past ? 0.f : ptx::ex2(s01.x);
+                    p[1] = past ? 0.f : ptx::ex2(s01.y);
+                    p[2] = past ? 0.f : ptx::ex2(s23.x);
+                    p[3] = past ? 0.f : ptx::ex2(s23.y);
+                    pmax = fmaxf(pmax, fmaxf(fmaxf(p[0], p[1]), fmaxf(p[2], p[3])));
                 }
-                if (!ptx::bar_and(kBarComputeAnd, kComputeThreads, fine)) {
+            }
+            const bool first = i == grp;
+            if (first || ptx::bar_popc(kBarGroup + grp, kGroupThreads, pmax > kLazyW || st >= lim || !ready) != 0) {
+                // move the references to the heads' running maxima and lim past the row scales
+                if (ready) {
+#pragma unroll
+                    for (int blk = 0; blk < NB; ++blk) {
+                        F2 s01, s23;
+                        scores(blk, s01, s23);
+                        float *p = p_k + 4 * blk;
+                        p[0] = past ? -INFINITY : s01.x;
+                        p[1] = past ? -INFINITY : s01.y;
+                        p[2] = past ? -INFINITY : s23.x;
+                        p[3] = past ? -INFINITY : s23.y;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float wm = warp_max(p[k]);
+                            if (lane == 0) sm.red[grp][q4][4 * blk + k] = wm;
+                        }
+                    }
+                    // row scales are non-negative: their bits order as the values do
+                    const float smx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(st)));
+                    if (lane == 0) sm.red[grp][q4][8] = smx;
+                    // every output MMA of the group so far is done (tile i's waits for these weights)
+                    if (!first) ready = wait(&sm.o_full[(i - 2) % kBuf], ((i - 2) / kBuf) & 1);
+                }
+                if (!ptx::bar_and(kBarGroup + grp, kGroupThreads, ready)) {
                     ok = false;
                     break;
                 }
-                float tmax[KHH];
-#pragma unroll
-                for (int k = 0; k < KHH; ++k) {
-                    tmax[k] = sm.red[sb][kQuarters * hh][k];
-#pragma unroll
-                    for (int w = 1; w < kQuarters; ++w)
-                        tmax[k] = fmaxf(tmax[k], sm.red[sb][kQuarters * hh + w][k]);
-                }
-                float smax = sm.red[sb][0][KHH];
-#pragma unroll
-                for (int w = 1; w < 4; ++w) smax = fmaxf(smax, sm.red[sb][w][KHH]);
+                const float smax = fmaxf(fmaxf(sm.red[grp][0][8], sm.red[grp][1][8]),
+                                         fmaxf(sm.red[grp][2][8], sm.red[grp][3][8]));
                 const int es_new =
                     smax > 0.f ? max(es, (int)((__float_as_uint(smax) >> 23) & 0xFFu) - 126) : es;
                 // O so far was taken with 2^(6 - es): bring it to 2^(6 - es_new)
                 const float shift = es_new > es && es > -1000 ? __uint_as_float((uint32_t)max(1, 127 + es - es_new) << 23)
                                                                : 1.f;
-                bool rescale = shift != 1.f;
-#pragma unroll
-                for (int k = 0; k < KHH; ++k) {
-                    const bool live = kAllLive || KHH * hh + k < G;
-                    const float mn = fmaxf(m[k], tmax[k]);
-                    alpha[k] = live ? ptx::ex2(m[k] - mn) : 1.f;
-                    m[k] = live ? mn : m[k];
-                    p_k[k] = ptx::ex2(s_k[k] - m[k]);
-                    lsum[k] *= alpha[k];
-                    rescale = rescale || alpha[k] != 1.f;
-                }
                 if (es_new != es) {
                     es = es_new;
                     pow2_from_exp(es + 2, sc, inv);
                     lim = __uint_as_float((uint32_t)max(1, min(254, es + 127)) << 23);
                 }
-                if (i >= 1 && rescale) {
-                    // every output MMA so far is done (tile i's waits for this warp's weights)
-                    if (observe(i - 1)) {
-                        ptx::tc_fence_after();
-                        float ov[Sh::HP];
-                        tmem_ldn<Sh::HP>(tmem + kColO + Sh::HP * hh + lane_base, ov);
-                        uint32_t ou[Sh::HP];
+                ptx::tc_fence_after();
 #pragma unroll
-                        for (int c = 0; c < Sh::HP; ++c)
-                            ou[c] = __float_as_uint(ov[c] * (alpha[c % KHH] * shift));
-                        tmem_stn<Sh::HP>(tmem + kColO + Sh::HP * hh + lane_base, ou);
-                        ptx::tmem_wait_st();
-                        ptx::tc_fence_before();
-                    } else {
-                        carried = false;
+                for (int blk = 0; blk < NB; ++blk) {
+                    float alpha[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int h = 4 * blk + k;
+                        const float mn = fmaxf(mref[h], fmaxf(fmaxf(sm.red[grp][0][h], sm.red[grp][1][h]),
+                                                              fmaxf(sm.red[grp][2][h], sm.red[grp][3][h])));
+                        alpha[k] = ptx::ex2(mref[h] - mn);
+                        p_k[h] = ptx::ex2(p_k[h] - mn);
+                        lsum[h] *= alpha[k];
+                    }
+                    if (!first) {
+                        float ov[16];
+                        const uint32_t oc = tmem + kColO + 32 * grp + 16 * blk + lane_base;
+                        ptx::tmem_ld16(oc, ov);
+                        uint32_t ou[16];
+#pragma unroll
+                        for (int c = 0; c < 16; ++c)
+                            ou[c] = __float_as_uint(ov[c] * (alpha[c & 3] * shift));
+                        tmem_st16(oc, ou);
                     }
                 }
+                ptx::tmem_wait_st();
+                // every warp has read the old references: the new ones take their place (the
+                // group's next barrier separates the maxima of two slow tiles the same way)
+                ptx::bar_sync(kBarGroup + grp, kGroupThreads);
+                if (q4 == 0 && lane < Sh::NH)
+                    mref[lane] = fmaxf(mref[lane], fmaxf(fmaxf(sm.red[grp][0][lane], sm.red[grp][1][lane]),
+                                                         fmaxf(sm.red[grp][2][lane], sm.red[grp][3][lane])));
+                ptx::bar_sync(kBarGroup + grp, kGroupThreads);
             }
-            const float sts = st * sc;
-            F2 x[KHH / 2];
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&sm.s_empty[sb]);
+            // W row of token t: 3 E4M3 terms of 4 heads a block (16 bytes, zero padded). Each term
+            // but the last is the value rounded to E4M3; the exact residual times 16 goes on.
+            // (the output MMAs of tile i - kBuf have read this weight buffer)
+            if (i >= kBuf) carried = wait(&sm.o_full[sb], (i / kBuf - 1) & 1);
+            if (!carried) continue;
+            const F2 sts = f2(st * sc, st * sc);
+            uint8_t *row = sm.p[sb] + (t >> 3) * Sh::GS + (t & 7) * 16;
 #pragma unroll
-            for (int e = 0; e < KHH / 2; ++e) {
-                const F2 p = f2(p_k[2 * e], p_k[2 * e + 1]);
-                const F2 l = add2(f2(lsum[2 * e], lsum[2 * e + 1]), p);
-                lsum[2 * e] = l.x;
-                lsum[2 * e + 1] = l.y;
-                x[e] = mul2(p, f2(sts, sts));
-            }
-            // W row of token t: 3 E4M3 terms of this warp's KHH heads (4 KHH bytes, zero
-            // padded). Each term but the last is the value rounded to E4M3; the exact residual
-            // times 16 goes on.
-            uint32_t w[kJp];
+            for (int blk = 0; blk < NB; ++blk) {
+                F2 x[2];
 #pragma unroll
-            for (int j = 0; j < kJp; ++j) {
-                uint32_t c2[KHH / 2];
-#pragma unroll
-                for (int e = 0; e < KHH / 2; ++e) {
-                    F2 v = x[e];
-                    if (j + 1 < kJp) {
-                        // (scalar: the compiler may simplify c - (c - x) and (h + k) - k when
-                        // they are written with packed operations, which breaks the rounding)
-                        v = f2(e4m3_round(v.x), e4m3_round(v.y));
-                        x[e] = mul2(sub2(x[e], v), f2(16.f, 16.f));   // exact
-                    }
-                    c2[e] = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(v.x, v.y), __NV_SATFINITE,
-                                                                __NV_E4M3);
+                for (int e = 0; e < 2; ++e) {
+                    const int h = 4 * blk + 2 * e;
+                    const F2 p = f2(p_k[h], p_k[h + 1]);
+                    const F2 l = add2(f2(lsum[h], lsum[h + 1]), p);
+                    lsum[h] = l.x;
+                    lsum[h + 1] = l.y;
+                    x[e] = mul2(p, sts);
                 }
-                if constexpr (KHH == 4) w[j] = c2[0] | (c2[1] << 16);
-                else w[j] = c2[0];
-            }
-            {
-                // the warp's first output column HP hh: 16-column block and byte within it
-                uint8_t *row = sm.p[pb] + (t >> 3) * Sh::GS + ((Sh::HP * hh) >> 4) * 128 +
-                               (t & 7) * 16 + ((Sh::HP * hh) & 15);
-                if constexpr (KHH == 4)
-                    *reinterpret_cast<uint4 *>(row) = make_uint4(w[0], w[1], w[2], 0u);
-                else
-                    *reinterpret_cast<uint2 *>(row) = make_uint2(w[0] | (w[1] << 16), w[2]);
+                uint32_t w[kJp];
+#pragma unroll
+                for (int j = 0; j < kJp; ++j) {
+                    uint32_t c2[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        F2 v = x[e];
+                        if (j + 1 < kJp) {
+                            // (scalar: the compiler may simplify c - (c - x) and (h + k) - k when
+                            // they are written with packed operations, which breaks the rounding)
+                            v = f2(e4m3_round(v.x), e4m3_round(v.y));
+                            x[e] = mul2(sub2(x[e], v), f2(16.f, 16.f));   // exact
+                        }
+                        c2[e] = (uint32_t)__nv_cvt_float2_to_fp8x2(make_float2(v.x, v.y), __NV_SATFINITE,
+                                                                    __NV_E4M3);
+                    }
+                    w[j] = c2[0] | (c2[1] << 16);
+                }
+                *reinterpret_cast<uint4 *>(row + blk * 128) = make_uint4(w[0], w[1], w[2], 0u);
             }
             // The output MMAs read whole 32-token steps of the tile: rows past the end of the
             // sequence hold stale bytes (possibly NaN codes), so zero them.
-            if (hh == 0 && !valid && t < ((nvalid + 31) & ~31)) {
-                uint4 *cr = reinterpret_cast<uint4 *>(sm.codes[s] + t * 128);
+            if (past && t < ((nvalid + 31) & ~31)) {
+                uint4 *cr = reinterpret_cast<uint4 *>(sm.codes[st_i] + t * 128);
 #pragma unroll
                 for (int c = 0; c < 8; ++c) cr[c] = make_uint4(0u, 0u, 0u, 0u);
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&sm.p_full[pb]);
-        }
-        // O = (O_0 + O_1 / 16 + O_2 / 256) * inv once every output MMA is done
-        float o[KHH];
-#pragma unroll
-        for (int k = 0; k < KHH; ++k) o[k] = 0.f;
-        if (ok && carried) {
-            if (observe(n_tiles - 1)) {
-                ptx::tc_fence_after();
-                float ov[Sh::HP];
-                tmem_ldn<Sh::HP>(tmem + kColO + Sh::HP * hh + lane_base, ov);
-                ptx::tc_fence_before();
-#pragma unroll
-                for (int k = 0; k < KHH; ++k)
-                    o[k] = fmaf(ov[2 * KHH + k], 1.f / 256.f, fmaf(ov[KHH + k], 1.f / 16.f, ov[k])) * inv;
-            } else {
-                carried = false;
+            if (lane == 0) ptx::mbar_arrive(&sm.p_full[sb]);
+            st_i += 2;
+            if (st_i >= kStages) {
+                st_i -= kStages;
+                st_ph ^= 1;
             }
         }
-
-        // the epilogue's barrier (the row sums) settles the last waits
+        // the group's last output MMAs, then the merge of the two groups' states (a group
+        // without a tile has an empty one)
+        ok = ok && carried;
+        const int last = n_tiles - 1 - ((n_tiles - 1 - grp) & 1);     // the group's last tile
+        if (ok && last >= 0) {
+            if (last >= 2) ok = wait(&sm.o_full[(last - 2) % kBuf], ((last - 2) / kBuf) & 1);
+            ok = ok && wait(&sm.o_full[last % kBuf], (last / kBuf) & 1);
+        }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
-            for (int k = 0; k < KHH; ++k) lsum[k] += __shfl_xor_sync(0xffffffffu, lsum[k], off);
-        const int rb = n_tiles & 1;
+            for (int h = 0; h < Sh::NH; ++h) lsum[h] += __shfl_xor_sync(0xffffffffu, lsum[h], off);
+        // (the barrier ahead keeps these writes behind the last slow tile's reads of red)
+        ptx::bar_sync(kBarGroup + grp, kGroupThreads);
         if (lane == 0) {
 #pragma unroll
-            for (int k = 0; k < KHH; ++k) sm.red[rb][warp][k] = lsum[k];
+            for (int h = 0; h < Sh::NH; ++h) sm.red[grp][q4][h] = lsum[h];
+            if (q4 == 0) sm.winv[grp] = inv;
         }
-        if (ptx::bar_and(kBarComputeAnd, kComputeThreads, ok && carried)) {
+        if (ptx::bar_and(kBarComputeAnd, kComputeThreads, ok)) {
+            ptx::tc_fence_after();
+            const bool two = n_tiles > 1;
+            // O = (O_0 + O_1 / 16 + O_2 / 256) * inv of head h of a group
+            auto group_o = [&](int gi, int h) {
+                const uint32_t oc = tmem + kColO + 32 * gi + 16 * (h >> 2) + (h & 3) + lane_base;
+                const float o0 = ptx::tmem_ld1(oc), o1 = ptx::tmem_ld1(oc + 4), o2 = ptx::tmem_ld1(oc + 8);
+                return fmaf(o2, 1.f / 256.f, fmaf(o1, 1.f / 16.f, o0)) * sm.winv[gi];
+            };
 #pragma unroll
-            for (int k = 0; k < KHH; ++k) {
-                const int h = KHH * hh + k;
+            for (int e = 0; e < KR; ++e) {
+                const int h = h1 + e;
                 if (h >= G) continue;
-                float lt = 0.f;
-#pragma unroll
-                for (int w = 0; w < 4; ++w) lt += sm.red[rb][kQuarters * hh + w][k];
-                const float val = o[k] / lt;
+                const float m0 = sm.mref[0][h], m1 = two ? sm.mref[1][h] : -INFINITY;
+                const float M = fmaxf(m0, m1);
+                const float w0 = ptx::ex2(m0 - M), w1 = two ? ptx::ex2(m1 - M) : 0.f;
+                float lt = w0 * ((sm.red[0][0][h] + sm.red[0][1][h]) + (sm.red[0][2][h] + sm.red[0][3][h]));
+                float o = w0 * group_o(0, h);
+                if (two) {
+                    lt += w1 * ((sm.red[1][0][h] + sm.red[1][1][h]) + (sm.red[1][2][h] + sm.red[1][3][h]));
+                    o += w1 * group_o(1, h);
+                }
+                const float val = o / lt;
                 const size_t bh = (size_t)b * geo.Hq + qh0 + h;
                 if (a.direct_out) {
                     if (a.out_dtype == KL_FP32) static_cast<float *>(a.out)[bh * kD + t] = val;
@@ -902,7 +846,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                     const size_t slot = bh * geo.S + split;
                     a.part_o[slot * kD + t] = val;
                     if (t == 0) {
-                        a.part_ml[slot * 2] = m[k] * kLn2;
+                        a.part_ml[slot * 2] = M * kLn2;
                         a.part_ml[slot * 2 + 1] = lt;
                     }
                 }
@@ -958,16 +902,15 @@ bool encode2d(CUtensorMap *map, CUtensorMapDataType type, const void *base, uint
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The decode for one head count per compute warp (2 for groups of up to 4 query heads, else 4)
-// and whether every compute warp's heads are real (groups of exactly 4 or 8).
-template <int KHH, bool kAllLive, bool kExact>
+// The decode for one operand shape (one block of 4 query heads, or two).
+template <int NB, bool kExact>
 cudaError_t launch_shape(const DecodeArgs &a, const CUtensorMap &cmap, const CUtensorMap &wmap,
                          const CUtensorMap &qmap, const float *v_scales) {
     const Geometry &g = a.geo;
     const size_t smem = sizeof(Smem8) + 1024;
     static PerDeviceOnce once;
     const cudaError_t e = once.run([&] {
-        return cudaFuncSetAttribute(decode_fp8_kernel<KHH, kAllLive, kExact>,
+        return cudaFuncSetAttribute(decode_fp8_kernel<NB, kExact>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
@@ -977,20 +920,15 @@ cudaError_t launch_shape(const DecodeArgs &a, const CUtensorMap &cmap, const CUt
     cfg.dynamicSmemBytes = smem;
     cfg.stream = a.stream;
     const OverlapAttr overlap(cfg);
-    return cudaLaunchKernelEx(&cfg, decode_fp8_kernel<KHH, kAllLive, kExact>, cmap, wmap, qmap, a,
-                              v_scales);
+    return cudaLaunchKernelEx(&cfg, decode_fp8_kernel<NB, kExact>, cmap, wmap, qmap, a, v_scales);
 }
 
 template <bool kExact>
 cudaError_t launch_waits(const DecodeArgs &a, const CUtensorMap &cmap, const CUtensorMap &wmap,
                          const CUtensorMap &qmap, const float *v_scales) {
-    const Geometry &g = a.geo;
-    // groups of more than 8 heads: blocks of 8 (and a last, smaller one)
-    if (g.G % 8 == 0) return launch_shape<4, true, kExact>(a, cmap, wmap, qmap, v_scales);
-    if (g.G > 8) return launch_shape<4, false, kExact>(a, cmap, wmap, qmap, v_scales);
-    if (g.G == 4) return launch_shape<2, true, kExact>(a, cmap, wmap, qmap, v_scales);
-    return g.G < 4 ? launch_shape<2, false, kExact>(a, cmap, wmap, qmap, v_scales)
-                   : launch_shape<4, false, kExact>(a, cmap, wmap, qmap, v_scales);
+    // groups of more than 8 heads: CTAs of 8 heads (and a last, smaller one)
+    return a.geo.G <= 4 ? launch_shape<1, kExact>(a, cmap, wmap, qmap, v_scales)
+                        : launch_shape<2, kExact>(a, cmap, wmap, qmap, v_scales);
 }
 
 }  // namespace
