@@ -7,24 +7,31 @@
 // 32 / 64, so 32 heads cost one CTA 770 cycles per tile where four sibling CTAs of 8 heads spend
 // 2500, against the 1460 cycles in which HBM delivers a tile to each SM.
 //
-// One CTA has the whole SM, so the tile chain (scores, softmax, weights) must overlap itself:
-// the compute warps form two groups, group 0 takes the even tiles and group 1 the odd ones. Each
-// group keeps its own softmax state (reference, sums and an O accumulator in TMEM), so the groups
-// meet only at the end, where their two states are merged like two splits. The output MMAs of
-// kFold tiles accumulate in TMEM; then the group adds that sum to its O (fp32 columns in TMEM,
-// rounded to nearest by the compute warps) and the next tile starts it over. (Left to the MMAs
-// for a whole run, the tensor core's truncating adds raised the fp32 output's error against 64
-// bits from 2.5e-6 to 4.8e-6 at 8192 tokens.) The rare tile that moves a reference rescales both.
+// Two layouts (NG softmax groups of 8 compute warps per CTA):
+//  NG = 2, one CTA per SM with a ring of 5 or 6 tiles: group 0 takes the even tiles and group 1
+//    the odd ones, so that the tile chain (scores, softmax, weights) overlaps itself. Each group
+//    keeps its own softmax state (reference, sums and an O accumulator in TMEM), so the groups
+//    meet only at the end, where their two states are merged like two splits.
+//  NG = 1, two CTAs per SM with a ring of 3 tiles, 16 heads: for launches of several waves, whose
+//    start-ups and last wave then overlap and share HBM.
+// The output MMAs of kFold tiles accumulate in TMEM; then the group adds that sum to its O (fp32
+// columns in TMEM, rounded to nearest by the compute warps) and the next tile starts it over.
+// (Left to the MMAs for a whole run, the tensor core's truncating adds raised the fp32 output's
+// error against 64 bits from 2.5e-6 to 4.8e-6 at 8192 tokens.) The rare tile that moves a
+// reference rescales both.
 //
-// Warps (608 threads): group i = warps 8 i .. 8 i + 7: warp w of a group reads TMEM lane quarter
-// w % 4 (thread = token of S and P, output dim of O) and takes the KH = NH / 2 heads KH (w / 4) ..;
-// then the producer, the score-MMA issuer (TMEM owner) and the output-MMA issuer.
+// Warps: group i = warps 8 i .. 8 i + 7: warp w of a group reads TMEM lane quarter w % 4 (thread =
+// token of S and P, output dim of O) and takes the KH = NH / 2 heads KH (w / 4) ..; then the
+// producer, the score-MMA issuer (TMEM owner) and the output-MMA issuer.
 //
-// Measured (back-to-back calls, 8192 tokens): 64 sequences of 128 heads over 8 value heads 252 ->
-// 189 us, 256 sequences of 32 heads over one value head 248 -> 113 us (HBM floors 158 and 80 us);
-// the rest is the last, partly filled wave of CTAs and each CTA's start. With 16 bytes of spills
-// per thread and tile more, the second case ran 158 us: the shared memory leaves next to no L1, so
-// the references live in shared memory and the weights are formed 8 heads at a time.
+// Measured (back-to-back calls, 8192 tokens): 64 sequences of 128 heads over 8 value heads 252 us
+// with sibling CTAs of 8 heads, 185 with NG = 2, 163 with NG = 1 (HBM floor 158); 256 sequences of
+// 32 heads over one value head 248 us with siblings, 129 with NG = 1 (two CTAs per tile, bound by
+// the ring's round trip), 105 with NH = 32 and NG = 2 (floor 80; the rest is the last, partly
+// filled wave). One sequence of 100000 tokens, 128 / 8 heads: 47.9 us with NG = 1, 39.8 with
+// NG = 2. Spills cost much, since the shared memory leaves next to no L1: 48 bytes more per thread
+// and tile took the second case from 121 to 158 us, so the references live in shared memory and
+// the weights are formed 8 heads at a time.
 //
 // Each wait is bounded as in kl_decode_tc_kernel.cuh.
 #include "kl_decode_tc_kernel.cuh"
@@ -32,12 +39,7 @@
 namespace kl {
 namespace {
 
-constexpr int kWideWarps = 16;                       // compute warps, 8 per group
-constexpr int kWideGroupThreads = 256;
-constexpr int kWideComputeThreads = kWideWarps * 32;
-constexpr int kWideProducer = kWideWarps, kWideMma = kWideWarps + 1, kWidePv = kWideWarps + 2;
-constexpr int kWideThreads = (kWideWarps + 3) * 32;
-constexpr uint32_t kWideTmemCols = 512;
+constexpr int kWideGroupThreads = 256;               // 8 compute warps per softmax group
 constexpr uint32_t kBarGroup = 3;                    // + group: vote of one group's warps
 constexpr int kFold = 4;                             // tiles of a group summed by the MMAs alone
 constexpr int kWideMaxRuns = 256;                    // states merged per (b, g, head block)
@@ -46,24 +48,39 @@ constexpr int kWideMaxRuns = 256;                    // states merged per (b, g,
 // only keeps everything far from overflow.
 constexpr float kWideLazy = 1024.f;
 
-template <int NH>
+// Warp roles and sizes for NH heads per CTA and NG softmax groups: NG = 2, one CTA per SM; NG = 1,
+// two CTAs per SM.
+template <int NH, int NG>
+struct Wide {
+    static constexpr int kStages = NG == 1 ? 3 : NH == 32 ? 5 : 6;
+    static constexpr int kWarps = 8 * NG;                // compute warps
+    static constexpr int kProducer = kWarps, kMma = kWarps + 1, kPv = kWarps + 2;
+    static constexpr int kThreads = (kWarps + 3) * 32;
+    static constexpr int kCtas = NG == 1 ? 2 : 1;        // per SM
+    static constexpr uint32_t kTmemCols = 512 / kCtas;
+};
+
+template <int NH, int NG>
 struct __align__(1024) WideSmem {
-    static constexpr int kStages = NH == 32 ? 5 : 6;
+    static constexpr int kStages = Wide<NH, NG>::kStages;
     uint8_t tiles[kStages][kTileBytes];              // as Smem<false>::tiles
     uint8_t qr[2 * 2 * NH * 128];                    // routed query [half][hi | lo rows][128 B]
-    uint8_t p[2][kTile * 2 * NH * 2];                // per group: [16 groups of 8 tokens]
+    uint8_t p[NG][kTile * 2 * NH * 2];               // per group: [16 groups of 8 tokens]
                                                      // [2 NH / 8 blocks][8 tokens][16 B]
-    float red[2][4][NH];                             // per group and lane quarter: maxima
-    float lred[2][4][NH];                            // ... row sums
-    float mref[2][NH];                               // per group: the heads' references (in
+    float red[NG][4][NH];                            // per group and lane quarter: maxima
+    float lred[NG][4][NH];                           // ... row sums
+    float mref[NG][NH];                              // per group: the heads' references (in
                                                      // shared memory to save registers)
     uint64_t full[kStages], empty[kStages];
-    uint64_t s_full[4], s_empty[4], p_full[2], o_full[2];
+    uint64_t s_full[2 * NG], s_empty[2 * NG], p_full[NG], o_full[NG];
     uint64_t qr_full, r_full, drain, drain2, merge_full;
     int is_last;
     uint32_t tmem_base;
     int abort;
 };
+// (228 KB per SM, of which each CTA takes 1 KB for the system)
+static_assert(sizeof(WideSmem<16, 1>) <= 228 * 1024 / 2 - 1024, "two CTAs per SM");
+static_assert(sizeof(WideSmem<32, 2>) <= 227 * 1024 && sizeof(WideSmem<16, 2>) <= 227 * 1024, "one");
 
 // 8 consecutive columns at `a` and at `b` of the thread's TMEM lane, one wait.
 __device__ __forceinline__ void tmem_ld_cols8(uint32_t a, uint32_t b, float (&x)[8], float (&y)[8]) {
@@ -142,21 +159,27 @@ __device__ __forceinline__ float warp_max_redux(float f) {
     return __int_as_float(k >= 0 ? k : k ^ 0x7FFFFFFF);
 }
 
-template <int NH, bool kExact>
-__global__ void __launch_bounds__(kWideThreads, 1)
+template <int NH, int NG, bool kExact>
+__global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
     decode_wide_kernel(const __grid_constant__ CUtensorMap vmap,
                        const __grid_constant__ CUtensorMap wmap,
                        const __grid_constant__ CUtensorMap qmap, const DecodeArgs a) {
-    using S = WideSmem<NH>;
-    constexpr int NS = S::kStages;
+    using S = WideSmem<NH, NG>;
+    using W = Wide<NH, NG>;
+    constexpr int NS = W::kStages, kWideWarps = W::kWarps, kWideComputeThreads = 32 * W::kWarps;
+    constexpr int kWideProducer = W::kProducer, kWideMma = W::kMma, kWidePv = W::kPv;
+    constexpr uint32_t kWideTmemCols = W::kTmemCols;
     constexpr int KH = NH / 2;                           // heads per compute warp
     constexpr int N = 2 * NH;                            // MMA columns: hi | lo
     constexpr uint32_t kQHalf = N * 128;                 // one 64-dim half of the query operand
     constexpr uint32_t kGroupBytes = N / 8 * 128;        // P: one group of 8 tokens
-    // TMEM columns: S[4] and the MMAs' sums O[2], N each; then each group's folded O, NH each
-    constexpr uint32_t kColS = 0, kColO = 4 * N, kColF = 6 * N;
-    extern __shared__ uint8_t smem_raw[];
-    S &sm = *reinterpret_cast<S *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // TMEM columns: two S buffers and the MMAs' sum O of each group, N each; then each group's
+    // folded O, NH each
+    constexpr uint32_t kColS = 0, kColO = 2 * NG * N, kColF = 3 * NG * N;
+    static_assert(kColF + NG * NH <= kWideTmemCols, "");
+    // (aligned by declaration: with two CTAs per SM there is no room for slack)
+    extern __shared__ __align__(1024) uint8_t smem_wide[];
+    S &sm = *reinterpret_cast<S *>(smem_wide);
 
     const Geometry &geo = a.geo;
     const int hb = blockIdx.x % geo.nhb, cta = blockIdx.x / geo.nhb;
@@ -175,12 +198,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             ptx::mbar_init(&sm.full[s], 1);
             ptx::mbar_init(&sm.empty[s], 1);
         }
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 2 * NG; ++i) {
             ptx::mbar_init(&sm.s_full[i], 1);
-            ptx::mbar_init(&sm.s_empty[i], kWideWarps / 2);
+            ptx::mbar_init(&sm.s_empty[i], 8);
         }
-        for (int i = 0; i < 2; ++i) {
-            ptx::mbar_init(&sm.p_full[i], kWideWarps / 2);
+        for (int i = 0; i < NG; ++i) {
+            ptx::mbar_init(&sm.p_full[i], 8);
             ptx::mbar_init(&sm.o_full[i], 1);
         }
         ptx::mbar_init(&sm.qr_full, kWideWarps);
@@ -191,7 +214,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         sm.abort = 0;
         ptx::fence_mbar_init();
     }
-    if (tid < 2 * NH) (&sm.mref[0][0])[tid] = -INFINITY;
+    if (tid < NG * NH) (&sm.mref[0][0])[tid] = -INFINITY;
     if (warp == kWideMma) {
         ptx::tmem_alloc(&sm.tmem_base, kWideTmemCols);
         ptx::tmem_relinquish();
@@ -383,9 +406,9 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         ok = ok && wait(&sm.qr_full, 0);
         if (ok) ptx::tc_fence_after();
         for (int i = 0; ok && i < n_tiles; ++i) {
-            const int r = i + ro, s = r % NS, sb = i & 3;
+            const int r = i + ro, s = r % NS, sb = i % (2 * NG);
             if (!wait(&sm.full[s], (r / NS) & 1)) break;
-            if (i >= 4 && !wait(&sm.s_empty[sb], ((i >> 2) - 1) & 1)) break;
+            if (i >= 2 * NG && !wait(&sm.s_empty[sb], (i / (2 * NG) - 1) & 1)) break;
             ptx::tc_fence_after();
             if (ptx::elect_one()) {
                 const uint64_t a0 = k_desc + ((s * kTileBytes) >> 4);
@@ -414,8 +437,8 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             ptx::smem_desc(ptx::smem_addr(sm.tiles[0]), kHalfBytes, 1024, ptx::kSwizzle128B);
         const uint64_t p_desc = ptx::smem_desc(ptx::smem_addr(sm.p[0]), kGroupBytes, 128, ptx::kSwizzleNone);
         for (int j = 0; j < n_tiles; ++j) {
-            const int s = (j + ro) % NS, pb = j & 1;
-            if (!wait(&sm.p_full[pb], (j >> 1) & 1)) break;
+            const int s = (j + ro) % NS, pb = j % NG, k = j / NG;
+            if (!wait(&sm.p_full[pb], k & 1)) break;
             ptx::tc_fence_after();
             const int nvalid = min(kTile, t_end - (t_begin + j * kTile));
             const int ksteps = (nvalid + 15) >> 4;
@@ -424,7 +447,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 const uint64_t b0 = p_desc + ((pb * sizeof(sm.p[0])) >> 4);
                 for (int kk = 0; kk < ksteps; ++kk)
                     ptx::mma_bf16(tmem + kColO + pb * N, a0 + ((kk * 2048) >> 4),
-                                  b0 + ((kk * 2 * kGroupBytes) >> 4), idesc_o, (j >> 1) % kFold != 0 || kk > 0);
+                                  b0 + ((kk * 2 * kGroupBytes) >> 4), idesc_o, k % kFold != 0 || kk > 0);
                 ptx::mma_commit(&sm.o_full[pb]);
                 ptx::mma_commit(&sm.empty[s]);
             }
@@ -437,15 +460,15 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         }
     } else {
         // ------------------------------------------------------------------ compute -----
-        const int grp = warp >> 3, qd = warp & 3, hs = (warp >> 2) & 1;
+        const int grp = NG == 2 ? warp >> 3 : 0, qd = warp & 3, hs = (warp >> 2) & 1;
         const int t = qd * 32 + lane;                   // token, and output dim
         const int h0 = KH * hs;
         const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
         bool ok = true;
 
-        // Routed query, thread = dim t: the two groups share the warp pair's KH heads between
-        // them (heads h1 .. h1 + KH / 2 - 1), split into hi and lo bf16 rows of the operand.
-        constexpr int KR = KH / 2;
+        // Routed query, thread = dim t: the groups share the warp pair's KH heads between them
+        // (heads h1 .. h1 + KR - 1 each), split into hi and lo bf16 rows of the operand.
+        constexpr int KR = KH / NG;
         const int h1 = h0 + KR * grp;
         if (route) {
             ok = wait(&sm.r_full, 0);
@@ -510,12 +533,12 @@ __global__ void __launch_bounds__(kWideThreads, 1)
         };
         bool carried = ok;
         ok = true;
-        for (int i = grp; i < n_tiles; i += 2) {
-            const int k = i >> 1, sb = i & 3;            // the group's tile count, S buffer
+        for (int i = grp; i < n_tiles; i += NG) {
+            const int k = i / NG, sb = i % (2 * NG);     // the group's tile count, S buffer
             const uint32_t sc = tmem + kColS + sb * N + h0 + lane_base;
             const int nvalid = min(kTile, t_end - (t_begin + i * kTile));
             const bool past = t >= nvalid;               // a token past the end: weight 0
-            bool ready = carried && wait(&sm.s_full[sb], (i >> 2) & 1);
+            bool ready = carried && wait(&sm.s_full[sb], (k >> 1) & 1);
             // the weights against the current references, 8 heads at a time
             float p[KH];
             float pmax = 0.f;
@@ -542,20 +565,19 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             bool freed = first;
             if (first || ptx::bar_popc(kBarGroup + grp, kWideGroupThreads, pmax > kWideLazy || !ready) != 0) {
                 // the per-head maximum over the tile's 128 tokens becomes the reference
+                if (ready) {
 #pragma unroll
-                for (int c = 0; c < KH; c += 8) {
-                    float hi[8], lo[8];
-                    if (ready) tmem_ld_cols8(sc + c, sc + NH + c, hi, lo);
+                    for (int c = 0; c < KH; c += 8) {
+                        float hi[8], lo[8];
+                        tmem_ld_cols8(sc + c, sc + NH + c, hi, lo);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        p[c + e] = past || !ready ? -INFINITY : hi[e] + lo[e];
-                        const float wm = warp_max_redux(p[c + e]);
-                        if (lane == e) sm.red[grp][qd][h0 + c + e] = wm;
+                        for (int e = 0; e < 8; ++e) {
+                            p[c + e] = past ? -INFINITY : hi[e] + lo[e];
+                            const float wm = warp_max_redux(p[c + e]);
+                            if (lane == e) sm.red[grp][qd][h0 + c + e] = wm;
+                        }
                     }
-                }
-                if (!first) {
-                    freed = ready && wait(&sm.o_full[grp], (k - 1) & 1);
-                    ready = ready && freed;
+                    if (!first) ready = freed = wait(&sm.o_full[grp], (k - 1) & 1);
                 }
                 if (!ptx::bar_and(kBarGroup + grp, kWideGroupThreads, ready)) {
                     ok = false;
@@ -610,7 +632,21 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&sm.s_empty[sb]);
-            // P^T row of token t, this warp's heads: hi and lo blocks of 8
+            // P^T row of token t, this warp's heads, hi and lo (formed before the wait: the MMAs that
+            // read the weight buffer are still running)
+            uint32_t ph[KH / 2], pl[KH / 2];
+#pragma unroll
+            for (int e = 0; e < KH / 2; ++e) {
+                const F2 pe = f2(p[2 * e], p[2 * e + 1]);
+                const F2 l = add2(f2(lsum[2 * e], lsum[2 * e + 1]), pe);
+                lsum[2 * e] = l.x;
+                lsum[2 * e + 1] = l.y;
+                const __nv_bfloat162 h2 = __floats2bfloat162_rn(pe.x, pe.y);
+                ph[e] = *reinterpret_cast<const uint32_t *>(&h2);
+                const F2 r = sub2(pe, f2(__uint_as_float(ph[e] << 16), __uint_as_float(ph[e] & 0xffff0000u)));
+                const __nv_bfloat162 l2 = __floats2bfloat162_rn(r.x, r.y);
+                pl[e] = *reinterpret_cast<const uint32_t *>(&l2);
+            }
             if (!freed) carried = wait(&sm.o_full[grp], (k - 1) & 1);
             if (carried) {
                 if (k % kFold == 0 && k > 0) {
@@ -623,24 +659,11 @@ __global__ void __launch_bounds__(kWideThreads, 1)
                 }
                 uint8_t *row = sm.p[grp] + (t >> 3) * kGroupBytes + (t & 7) * 16 + (h0 >> 3) * 128;
 #pragma unroll
-                for (int c = 0; c < KH; c += 8) {
-                    uint32_t ph[4], pl[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const F2 pe = f2(p[c + 2 * e], p[c + 2 * e + 1]);
-                        const F2 l = add2(f2(lsum[c + 2 * e], lsum[c + 2 * e + 1]), pe);
-                        lsum[c + 2 * e] = l.x;
-                        lsum[c + 2 * e + 1] = l.y;
-                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(pe.x, pe.y);
-                        ph[e] = *reinterpret_cast<const uint32_t *>(&h2);
-                        const F2 r = sub2(pe, f2(__uint_as_float(ph[e] << 16),
-                                                 __uint_as_float(ph[e] & 0xffff0000u)));
-                        const __nv_bfloat162 l2 = __floats2bfloat162_rn(r.x, r.y);
-                        pl[e] = *reinterpret_cast<const uint32_t *>(&l2);
-                    }
-                    *reinterpret_cast<uint4 *>(row + (c >> 3) * 128) = make_uint4(ph[0], ph[1], ph[2], ph[3]);
-                    *reinterpret_cast<uint4 *>(row + ((NH + c) >> 3) * 128) =
-                        make_uint4(pl[0], pl[1], pl[2], pl[3]);
+                for (int c = 0; c < KH / 8; ++c) {
+                    *reinterpret_cast<uint4 *>(row + c * 128) =
+                        make_uint4(ph[4 * c], ph[4 * c + 1], ph[4 * c + 2], ph[4 * c + 3]);
+                    *reinterpret_cast<uint4 *>(row + (NH / 8 + c) * 128) =
+                        make_uint4(pl[4 * c], pl[4 * c + 1], pl[4 * c + 2], pl[4 * c + 3]);
                 }
                 // rows past the end inside the last 16-token MMA step must be finite: zero them
                 // (each of the lane quarter's two warps one 64-dim half)
@@ -659,7 +682,7 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             }
         }
         // the group's last output MMAs (a group without a tile has an empty state)
-        const int mine = (n_tiles + 1 - grp) >> 1;
+        const int mine = (n_tiles + NG - 1 - grp) / NG;
         ok = ok && carried;
         if (ok && mine > 0) ok = wait(&sm.o_full[grp], (mine - 1) & 1);
 #pragma unroll
@@ -678,26 +701,47 @@ __global__ void __launch_bounds__(kWideThreads, 1)
             // one run of the whole sequence writes the output, else the run's state
             const int n_cta_u = (L + geo.chunk * geo.spc - 1) / (geo.chunk * geo.spc);
             const bool write_out = a.direct_out || n_cta_u == 1;
-            const bool two = n_tiles > 1;
-            const int mine0 = (n_tiles + 1) >> 1;
-            // O of head h of a group that ran n tiles: the folded sum and the MMAs' last one
-            auto group_o = [&](int gi, int h, int n) {
-                const uint32_t oc = tmem + kColO + gi * N + h + lane_base;
-                const float o = ptx::tmem_ld1(oc) + ptx::tmem_ld1(oc + NH);
-                return n > kFold ? o + ptx::tmem_ld1(tmem + kColF + gi * NH + h + lane_base) : o;
+            const bool two = NG == 2 && n_tiles > 1;
+            const int mine0 = (n_tiles + NG - 1) / NG;
+            // O of heads h1 .. h1 + KR - 1 of a group that ran n tiles: the folded sum and the MMAs'
+            // last one
+            auto group_o = [&](int gi, int n, float (&o)[KR]) {
+                const uint32_t oc = tmem + kColO + gi * N + h1 + lane_base;
+                const uint32_t fc = tmem + kColF + gi * NH + h1 + lane_base;
+                if constexpr (KR == 8) {
+                    float lo[8];
+                    tmem_ld_cols8(oc, oc + NH, o, lo);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) o[e] += lo[e];
+                    if (n > kFold) {
+                        tmem_ld_col8(fc, lo);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) o[e] += lo[e];
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < KR; ++e) {
+                        o[e] = ptx::tmem_ld1(oc + e) + ptx::tmem_ld1(oc + NH + e);
+                        if (n > kFold) o[e] += ptx::tmem_ld1(fc + e);
+                    }
+                }
             };
+            float o0[KR], o1[KR];
+            group_o(0, mine0, o0);
+            if (two) group_o(NG - 1, n_tiles >> 1, o1);
 #pragma unroll
             for (int e = 0; e < KR; ++e) {
                 const int h = h1 + e;
                 if (h >= G) continue;
-                const float m0 = sm.mref[0][h], m1 = two ? sm.mref[1][h] : -INFINITY;
+                const float m0 = sm.mref[0][h], m1 = two ? sm.mref[NG - 1][h] : -INFINITY;
                 const float M = fmaxf(m0, m1);
                 const float w0 = ptx::ex2(m0 - M), w1 = two ? ptx::ex2(m1 - M) : 0.f;
                 float lt = w0 * ((sm.lred[0][0][h] + sm.lred[0][1][h]) + (sm.lred[0][2][h] + sm.lred[0][3][h]));
-                float o = w0 * group_o(0, h, mine0);
+                float o = w0 * o0[e];
                 if (two) {
-                    lt += w1 * ((sm.lred[1][0][h] + sm.lred[1][1][h]) + (sm.lred[1][2][h] + sm.lred[1][3][h]));
-                    o += w1 * group_o(1, h, n_tiles >> 1);
+                    const auto &l1 = sm.lred[NG - 1];
+                    lt += w1 * ((l1[0][h] + l1[1][h]) + (l1[2][h] + l1[3][h]));
+                    o += w1 * o1[e];
                 }
                 const float val = o / lt;
                 const size_t bh = (size_t)b * geo.Hq + qh0 + h;
@@ -743,24 +787,31 @@ __global__ void __launch_bounds__(kWideThreads, 1)
     }
 }
 
-template <int NH, bool kExact>
-cudaError_t launch_wide(const DecodeArgs &la, const CUtensorMap &vmap, const CUtensorMap &wmap,
-                        const CUtensorMap &qmap) {
+template <int NH, int NG, bool kExact>
+cudaError_t launch_kernel_wide(const DecodeArgs &la, const CUtensorMap &vmap, const CUtensorMap &wmap,
+                               const CUtensorMap &qmap) {
     const Geometry &g = la.geo;
-    const size_t smem = sizeof(WideSmem<NH>) + 1024;
+    const size_t smem = sizeof(WideSmem<NH, NG>);
     static PerDeviceOnce once;
     const cudaError_t e = once.run([&] {
-        return cudaFuncSetAttribute(decode_wide_kernel<NH, kExact>,
+        return cudaFuncSetAttribute(decode_wide_kernel<NH, NG, kExact>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((g.S + g.spc - 1) / g.spc * g.nhb, g.Hkv, g.B);
-    cfg.blockDim = dim3(kWideThreads);
+    cfg.blockDim = dim3(Wide<NH, NG>::kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = la.stream;
     const OverlapAttr overlap(cfg);
-    return cudaLaunchKernelEx(&cfg, decode_wide_kernel<NH, kExact>, vmap, wmap, qmap, la);
+    return cudaLaunchKernelEx(&cfg, decode_wide_kernel<NH, NG, kExact>, vmap, wmap, qmap, la);
+}
+
+template <int NH, int NG>
+cudaError_t launch_wide(const DecodeArgs &la, const CUtensorMap &vmap, const CUtensorMap &wmap,
+                        const CUtensorMap &qmap) {
+    return la.wait_ns < kExactWaitNs ? launch_kernel_wide<NH, NG, true>(la, vmap, wmap, qmap)
+                                     : launch_kernel_wide<NH, NG, false>(la, vmap, wmap, qmap);
 }
 
 }  // namespace
@@ -768,17 +819,22 @@ cudaError_t launch_wide(const DecodeArgs &la, const CUtensorMap &vmap, const CUt
 cudaError_t launch_tc_wide(const DecodeArgs &a) {
     DecodeArgs la = a;
     Geometry &g = la.geo;
-    const int64_t slots = device_sm_count();
+    const int64_t sms = device_sm_count();
     // 32 heads per CTA read each tile once for a group of 17 or more; with fewer such CTAs than
     // SMs, blocks of 16 spread the group over twice as many.
-    const int nh32 = (g.G + 31) / 32;
-    const bool w32 = g.G > 16 && (int64_t)g.B * g.Hkv * nh32 * g.S >= slots;
+    const int64_t units8 = (int64_t)g.B * g.Hkv;
+    const bool w32 = g.G > 16 && units8 * ((g.G + 31) / 32) * g.S >= sms;
     const int NH = w32 ? 32 : 16;
     g.nhb = (g.G + NH - 1) / NH;
     g.qbox = g.G < NH ? g.G : NH;
+    // Blocks of 16 heads that overflow one CTA per SM go two to an SM with one softmax group each:
+    // their waves overlap, and the last one shares HBM evenly. (Within one wave, the
+    // deeper ring and the two groups of a CTA that has its SM alone are faster.)
+    const int64_t units = units8 * g.nhb;
+    const bool two_per_sm = !w32 && units > sms;
+    const int64_t slots = two_per_sm ? 2 * sms : sms;
     // consecutive splits per CTA: the fewest that fit one wave (when the units alone do not fill
     // it), and at most kWideMaxRuns states to merge
-    const int64_t units = (int64_t)g.B * g.Hkv * g.nhb;
     int spc = (g.S + kWideMaxRuns - 1) / kWideMaxRuns;
     if (g.S > 1 && units < slots)
         while ((int64_t)((g.S + spc - 1) / spc) * units > slots) ++spc;
@@ -793,10 +849,8 @@ cudaError_t launch_tc_wide(const DecodeArgs &a) {
         if (!make_map(&qmap, a.q, kD, (uint64_t)g.B * g.Hq, (uint32_t)g.qbox))
             return cudaErrorInvalidValue;
     }
-    const bool exact = a.wait_ns < kExactWaitNs;
-    if (w32)
-        return exact ? launch_wide<32, true>(la, vmap, wmap, qmap) : launch_wide<32, false>(la, vmap, wmap, qmap);
-    return exact ? launch_wide<16, true>(la, vmap, wmap, qmap) : launch_wide<16, false>(la, vmap, wmap, qmap);
+    if (w32) return launch_wide<32, 2>(la, vmap, wmap, qmap);
+    return two_per_sm ? launch_wide<16, 1>(la, vmap, wmap, qmap) : launch_wide<16, 2>(la, vmap, wmap, qmap);
 }
 
 }  // namespace kl
