@@ -73,11 +73,12 @@ constexpr int kProducerWarp = 8;
 constexpr int kMmaWarp = 9;
 constexpr int kPvWarp = 10;
 constexpr int kThreads = 11 * 32;
-constexpr int kStages = 5;
+constexpr int kStages = 6;
 constexpr uint32_t kCodeBytes = kTile * kD;          // 16 KiB of codes per tile
 constexpr uint32_t kHalfBytes = 16384;               // one 64-column half of W^R (bf16)
 constexpr uint32_t kPBytes = 4096;                   // weight operand buffer (largest shape)
-constexpr int kBuf = 4;                              // score and weight buffers, two per group
+constexpr int kBuf = 4;                              // score buffers, two per group (and one
+                                                     // weight buffer each)
 constexpr uint32_t kTmemCols = 256;
 constexpr uint32_t kColS = 0;                        // S[b]: columns 32 b .. 32 b + 31
 constexpr uint32_t kColO = 128;                      // O of group i: 128 + 32 i .., summed over
@@ -108,7 +109,7 @@ struct __align__(1024) Smem8 {
     // Weight terms, B operand of the output MMAs: [16 groups of 8 tokens][N / 16 blocks of 16
     // columns][8 tokens][16 B], MN-major, no swizzle. During the routing prologue the first one
     // holds the query rows: [64-dim half][16 rows][128 B], K-major, 128B-swizzled.
-    uint8_t p[kBuf][kPBytes];
+    uint8_t p[2][kPBytes];
     float scl[kStages][kTile];         // row scales of each stage's tile, token order
     float red[2][4][12];               // per group and lane quarter: 8 head maxima (or row sums),
                                        // then the scale maximum
@@ -116,7 +117,7 @@ struct __align__(1024) Smem8 {
     float invq[8];                     // per head: the inverse power of its query terms
     float winv[2];                     // per group: the inverse power of its weights
     uint64_t full[kStages], empty[kStages];
-    uint64_t s_full[kBuf], s_empty[kBuf], p_full[kBuf], o_full[kBuf];
+    uint64_t s_full[kBuf], s_empty[kBuf], p_full[2], o_full[2];
     uint64_t r_full, qt_full, drain, drain2;
     uint32_t tmem_base;
     int abort;
@@ -271,6 +272,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&u)[16
         : "memory");
 }
 
+// two CTAs per SM: 228 KB, of which each CTA takes 1 KB for the system
+static_assert(sizeof(Smem8) + 1024 <= 228 * 1024 / 2 - 1024, "two CTAs per SM");
+
 template <int NB, bool kExact>
 __global__ void __launch_bounds__(kThreads, 2)
     decode_fp8_kernel(const __grid_constant__ CUtensorMap cmap,
@@ -302,6 +306,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         for (int i = 0; i < kBuf; ++i) {
             ptx::mbar_init(&sm.s_full[i], 1);
             ptx::mbar_init(&sm.s_empty[i], kComputeWarps / 2);
+        }
+        for (int i = 0; i < 2; ++i) {
             ptx::mbar_init(&sm.p_full[i], kComputeWarps / 2);
             ptx::mbar_init(&sm.o_full[i], 1);
         }
@@ -520,8 +526,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         const uint64_t p_desc =
             ptx::smem_desc(ptx::smem_addr(sm.p[0]), Sh::GS, 128, ptx::kSwizzleNone);
         for (int j = 0; j < n_tiles; ++j) {
-            const int u = j + base, s = u % kStages, pb = j % kBuf;
-            if (!wait(&sm.p_full[pb], (j / kBuf) & 1)) break;
+            const int u = j + base, s = u % kStages, pb = j & 1;
+            if (!wait(&sm.p_full[pb], (j >> 1) & 1)) break;
             ptx::tc_fence_after();
             const int nvalid = min(kTile, t_end - (t_begin + j * kTile));
             const int ksteps = (nvalid + 31) >> 5;
@@ -529,9 +535,9 @@ __global__ void __launch_bounds__(kThreads, 2)
                 const uint64_t a0 = c_desc + ((s * kCodeBytes) >> 4);
                 const uint64_t b0 = p_desc + ((pb * kPBytes) >> 4);
                 for (int kk = 0; kk < ksteps; ++kk)
-                    mma_f8(tmem + kColO + (j & 1) * 32, a0 + ((kk * 4096) >> 4),
+                    mma_f8(tmem + kColO + pb * 32, a0 + ((kk * 4096) >> 4),
                            b0 + ((kk * 4 * Sh::GS) >> 4), idesc_o, (j > 1 || kk > 0) ? 1u : 0u);
-                ptx::mma_commit(&sm.o_full[pb]);   // tile j: phase j / kBuf of o_full[j % kBuf]
+                ptx::mma_commit(&sm.o_full[pb]);
                 ptx::mma_commit(&sm.empty[s]);     // the tile's last reader is done
             }
             __syncwarp();
@@ -687,7 +693,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                     const float smx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(st)));
                     if (lane == 0) sm.red[grp][q4][8] = smx;
                     // every output MMA of the group so far is done (tile i's waits for these weights)
-                    if (!first) ready = wait(&sm.o_full[(i - 2) % kBuf], ((i - 2) / kBuf) & 1);
+                    if (!first) ready = wait(&sm.o_full[grp], ((i >> 1) - 1) & 1);
                 }
                 if (!ptx::bar_and(kBarGroup + grp, kGroupThreads, ready)) {
                     ok = false;
@@ -743,11 +749,11 @@ __global__ void __launch_bounds__(kThreads, 2)
             if (lane == 0) ptx::mbar_arrive(&sm.s_empty[sb]);
             // W row of token t: 3 E4M3 terms of 4 heads a block (16 bytes, zero padded). Each term
             // but the last is the value rounded to E4M3; the exact residual times 16 goes on.
-            // (the output MMAs of tile i - kBuf have read this weight buffer)
-            if (i >= kBuf) carried = wait(&sm.o_full[sb], (i / kBuf - 1) & 1);
+            // (the output MMAs of the group's previous tile have read the weight buffer)
+            if (i >= 2) carried = wait(&sm.o_full[grp], ((i >> 1) - 1) & 1);
             if (!carried) continue;
             const F2 sts = f2(st * sc, st * sc);
-            uint8_t *row = sm.p[sb] + (t >> 3) * Sh::GS + (t & 7) * 16;
+            uint8_t *row = sm.p[grp] + (t >> 3) * Sh::GS + (t & 7) * 16;
 #pragma unroll
             for (int blk = 0; blk < NB; ++blk) {
                 F2 x[2];
@@ -789,7 +795,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             }
             ptx::fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(&sm.p_full[sb]);
+            if (lane == 0) ptx::mbar_arrive(&sm.p_full[grp]);
             st_i += 2;
             if (st_i >= kStages) {
                 st_i -= kStages;
@@ -799,11 +805,8 @@ __global__ void __launch_bounds__(kThreads, 2)
         // the group's last output MMAs, then the merge of the two groups' states (a group
         // without a tile has an empty one)
         ok = ok && carried;
-        const int last = n_tiles - 1 - ((n_tiles - 1 - grp) & 1);     // the group's last tile
-        if (ok && last >= 0) {
-            if (last >= 2) ok = wait(&sm.o_full[(last - 2) % kBuf], ((last - 2) / kBuf) & 1);
-            ok = ok && wait(&sm.o_full[last % kBuf], (last / kBuf) & 1);
-        }
+        const int mine = (n_tiles + 1 - grp) >> 1;                 // the group's tiles
+        if (ok && mine > 0) ok = wait(&sm.o_full[grp], (mine - 1) & 1);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
