@@ -83,6 +83,9 @@ struct PrefillArgs {
     Geometry geo;             // S and chunk unused
     int total_q;              // rows of q and out
     int max_q;                // host bound on n_b (grid sizing)
+    // Layout (set by the launcher): a block of 128 rows holds hp heads of one value head's group,
+    // rpb query rows each; a cluster of cs CTAs splits a block's cache tiles.
+    int hp = 1, rpb = 128, cs = 1;
     const uint16_t *q;        // [total_q][Hq][D] bf16
     const uint16_t *w_r;      // [Hw][D][D] bf16
     const uint16_t *v_cache;  // [num_pages][Hkv][P][D] bf16
@@ -114,14 +117,14 @@ __device__ __forceinline__ void grid_dep_launch() {
 }
 
 // Launch attribute of every kernel here: a programmatic dependent of the kernel ahead of it in the
-// stream. Where that kernel signals early (these kernels do, once all of their CTAs run), the
-// launch latency and the set-up overlap its end; each kernel calls grid_dep_wait() in all threads
-// before its first access to global memory (through pointers without __restrict__, whose loads
-// the compiler may not move above the wait), so stream order holds for everything it reads and
-// writes, and signals only once it holds its tensor memory, so that no CTA that waits for it can
-// take that. Behind any other kernel it starts as an ordinary launch. Calls one after another:
-// 8 x 4096 tokens 20.0 -> 16.9 us, one sequence of 131072 49.4 -> 47.0 us, 32 x 8192 at head dim
-// 64 86.2 -> 81.9 us, the 70B batch 604 -> 594 us.
+// stream. Where that kernel signals early (these kernels but the prefill do, once all of their
+// CTAs run), the launch latency and the set-up overlap its end; each kernel calls grid_dep_wait()
+// in all threads before its first access to global memory (through pointers without __restrict__,
+// whose loads the compiler may not move above the wait), so stream order holds for everything it
+// reads and writes, and signals only once it holds its tensor memory, so that no CTA that waits
+// for it can take that. Behind any other kernel it starts as an ordinary launch. Calls one after
+// another: 8 x 4096 tokens 20.0 -> 16.9 us, one sequence of 131072 49.4 -> 47.0 us, 32 x 8192 at
+// head dim 64 86.2 -> 81.9 us, the 70B batch 604 -> 594 us.
 struct OverlapAttr {
     cudaLaunchAttribute attr[1];
     explicit OverlapAttr(cudaLaunchConfig_t &cfg) {

@@ -4,6 +4,10 @@
 // One CTA per (query head h, sequence b, block of 128 query rows); head_dim 128. The rows of the
 // block sit at consecutive positions p0 .. p0 + 127 of the sequence (the chunk is the tail of the
 // cached rows), so the CTA walks the cache tiles 0 .. p_last / 128 and masks only the last ones.
+// Small chunks share more (kShared): a block's 128 rows hold several heads of a group, which read
+// the same tiles, and while the blocks leave SMs idle, a cluster of up to 8 CTAs splits a block's
+// tiles and merges the states through distributed shared memory. (4 sequences of 4000 tokens,
+// 16-token chunks, 12 heads: 43 -> 27 us; 2 of 8000 tokens, 100-token chunks, 32 heads: 85 -> 56.)
 //
 //   routing  Q_r = Q . W^R[w(h)]                      M = 128 rows, N = 128, K = 128 (Section 2.2)
 //   scores   S   = Q_hi . V_t^T + Q_lo . V_t^T        M = 128 rows, N = 128 tokens, K = 2 x 128
@@ -101,6 +105,7 @@ struct __align__(1024) PrefillSmem {
     uint64_t r_full, qr_ready, drain, drain2;
     float mref[2][kBM];        // the rows' references after the last half tile of each parity
     float lsum[2][kBM];        // the two groups' shares of the row sums, for the epilogue
+    float2 ml[kBM];            // the rows' references and sums, for the cluster's merge
     uint32_t tmem_base;
     int abort;
 };
@@ -203,6 +208,9 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
                  : "memory");
 }
 
+// kShared: several heads per block or CTAs per cluster (a.hp, a.rpb, a.cs); otherwise one head per
+// block and one CTA per block, as constants.
+template <bool kShared>
 __global__ void __launch_bounds__(kThreads, 1)
     prefill_tc_kernel(const __grid_constant__ CUtensorMap vmap,
                       const __grid_constant__ CUtensorMap wmap,
@@ -211,7 +219,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     PrefillSmem &sm = *reinterpret_cast<PrefillSmem *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const Geometry &geo = a.geo;
-    const int h = blockIdx.x, b = blockIdx.y;
+    const int cs = kShared ? a.cs : 1, hp = kShared ? a.hp : 1, rpb = kShared ? a.rpb : kBM;
+    const int rank = blockIdx.x % cs, hg = blockIdx.x / cs, b = blockIdx.y;
     const int mblk = (int)gridDim.z - 1 - (int)blockIdx.z;   // the longest blocks start first
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -220,18 +229,28 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int L = a.seq_lens[b];
     const int n = q1 - q0;
     if (q0 < 0 || n < 0 || q1 > a.total_q || L < n || L > geo.max_pages * geo.P) {
-        if (tid == 0 && h == 0 && mblk == 0) raise_flag(a.err, KL_FLAG_BAD_LENGTH);
+        if (tid == 0 && blockIdx.x == 0 && mblk == 0) raise_flag(a.err, KL_FLAG_BAD_LENGTH);
         return;
     }
-    const int m0 = mblk * kBM;
+    // The block: query rows m0 .. m0 + rows - 1 of the chunk, heads h .. h + hn - 1; row r of the
+    // 128 is query row r / hp of head r % hp.
+    const int m0 = mblk * rpb;
     if (m0 >= n) return;
-    const int rows = min(kBM, n - m0);           // query rows of this block
+    const int rows = min(rpb, n - m0);
+    const int nhg = (geo.G + hp - 1) / hp;       // blocks of heads per value head
+    const int g = hg / nhg, h = g * geo.G + (hg % nhg) * hp;
+    const int hn = min(hp, (g + 1) * geo.G - h);
+    const int wsel = geo.wr_per_qh ? h : g;      // (one W^R per query head: hp is 1)
     const int pos0 = L - n + m0;                 // position of row 0
     const int pos_last = pos0 + rows - 1;        // <= L - 1
-    const int n_tiles = pos_last / kBN + 1;      // cache tiles 0 .. n_tiles - 1
-    const int n_sub = pos_last / kBS + 1;        // half tiles 0 .. n_sub - 1
-    const int g = h / geo.G;
-    const int wsel = geo.wr_per_qh ? h : g;
+    // The cluster's CTAs take consecutive shares of the block's cache tiles; this one's are tiles
+    // tile0 .. tile0 + n_tiles - 1, half tiles 0 .. n_sub - 1 from there (none for the last ranks
+    // of a short sequence).
+    const int all_tiles = pos_last / kBN + 1;
+    const int share = (all_tiles + cs - 1) / cs;
+    const int tile0 = min(all_tiles, rank * share);
+    const int n_tiles = min(share, all_tiles - tile0);
+    const int n_sub = max(0, min(2 * n_tiles, pos_last / kBS + 1 - 2 * tile0));
 
     if (tid == 0) {
         for (int s = 0; s < kStages; ++s) {
@@ -261,6 +280,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         ptx::tmem_alloc(&sm.tmem_base, kTmemCols);
         ptx::tmem_relinquish();
     }
+    // rows of the query block that its box does not fill
+    if (kShared) {
+        for (int i = tid; i < (kBM - hp * rpb) * 16; i += kThreads)
+            *reinterpret_cast<uint4 *>(sm.q + (i & 8 ? kHalfBytes : 0) + (hp * rpb + (i >> 4)) * 128 +
+                                       (i & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+        ptx::fence_proxy_async_smem();
+    }
     if (warp == kProducerWarp && lane == 0) {
         ptx::prefetch_tensormap(&vmap);
         ptx::prefetch_tensormap(&wmap);
@@ -269,13 +295,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    // the kernel behind may start setting up once every CTA is here (and holds its TMEM)
-    grid_dep_launch();
+    // (No early signal to the kernel behind: a chunk append that came to sit under the last wave
+    // made batches of short sequences slower, 16 x 16 heads of 100 to 3000 tokens 203 -> 230 us.)
 
     const uint32_t tmem = sm.tmem_base;
     const Waiter wait{&sm.abort, a.err};
 
-    if (warp == kProducerWarp) {
+    const int qd = warp & 3, hf = warp >> 2;     // softmax warps: lane quarter and group
+    const int r = qd * 32 + lane;                // query row = TMEM lane
+    if (kShared && n_sub == 0) {
+        // no share of the cache: an empty state
+        if (warp < 4) sm.ml[r] = make_float2(-INFINITY, 0.f);
+    } else if (warp == kProducerWarp) {
         // ------------------------------------------------------------------ producer ----
         const int P = geo.P;
         const int ppt = kBN / P;                          // pages per tile (<= 8)
@@ -286,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool bad = false;
         // position 0: W^R[w(h)] (B operand of the routing MMA) and the query block
         if (lane == 0) {
-            ptx::mbar_arrive_expect_tx(&sm.full[0], kTileBytes + kBM * kD * 2);
+            ptx::mbar_arrive_expect_tx(&sm.full[0], kTileBytes + hp * rpb * kD * 2);
             ptx::tma_load_2d(sm.tiles[0], &wmap, &sm.full[0], 0, wsel * kD);
             ptx::tma_load_2d(sm.tiles[0] + kHalfBytes, &wmap, &sm.full[0], 64, wsel * kD);
             ptx::tma_load_3d(sm.q, &qmap, &sm.full[0], 0, h, q0 + m0);
@@ -296,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         issued = 1;
         for (int i = 0; i < n_tiles; ++i) {
             const int r = i + 1, s = r % kStages;
-            const int pg = i * ppt + lane;                // page index within the sequence
+            const int pg = (tile0 + i) * ppt + lane;      // page index within the sequence
             const bool exists = lane < ppt && pg < seq_pages;
             const int page = exists ? bt[pg] : -1;
             if (r >= kStages && !wait(&sm.empty[s], ((r / kStages) & 1) ^ 1)) break;
@@ -411,13 +442,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         // around it. The groups share each row's reference (and O): the owner of half tile u takes
         // the reference that u - 1 left, and passes its own on (turn) before its exponentials. In
         // the prologue and the epilogue the two warps of a lane quarter split the 128 columns.
-        const int qd = warp & 3, hf = warp >> 2;
-        const int r = qd * 32 + lane;                        // query row = TMEM lane
         const int c0 = hf * 64;                              // this warp's columns
         const uint32_t lane_base = (uint32_t)(qd * 32) << 16;
         const uint32_t pair_bar = 1 + qd;
         // rows past the block's end take the last valid position: finite, never stored
-        const int pos_r = min(pos0 + r, pos_last);
+        const int pos_r = min(pos0 + r / hp, pos_last);
         const float sl2 = geo.scale * kLog2e;
         bool ok = wait(&sm.r_full, 0);
 
@@ -452,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
         bool okl = ok;
         for (int u = hf; okl && u < n_sub; u += 2) {
-            const int t0 = u * kBS, k = u >> 1, sb = u % kSub;
+            const int t0 = tile0 * kBN + u * kBS, k = u >> 1, sb = u % kSub;
             const uint32_t sbuf = tmem + kColS + (uint32_t)sb * kBS + lane_base;   // S, then P
             // This thread's half (64 dims) of a cache row of the half tile as fp16, formed while
             // the scores are still on their way: the output MMAs read the tile as fp16. Rows at
@@ -588,19 +617,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             l = m_used == -INFINITY ? 0.f : l * ptx::ex2(m_used - m_fin);
         }
         sm.lsum[hf][r] = l;
-        if (ptx::bar_and(pair_bar, 64, oke)) {
+        const bool okp = ptx::bar_and(pair_bar, 64, oke);
+        const float lt = l + sm.lsum[hf ^ 1][r];
+        if (kShared && cs > 1) {
+            if (hf == 0) sm.ml[r] = okp ? make_float2(sm.mref[lb2][r], lt) : make_float2(-INFINITY, 0.f);
+        } else if (okp) {
             ptx::tc_fence_after();
-            const float lt = l + sm.lsum[hf ^ 1][r];
             const float inv = lt > 0.f ? 1.f / lt : 0.f;
             float nf = 0.f;   // x * 0 is NaN exactly when x is not finite
-            const size_t orow = ((size_t)(q0 + m0 + r) * geo.Hq + h) * kD + c0;
+            const int ri = r / hp, hh = r - ri * hp;
+            const size_t orow = ((size_t)(q0 + m0 + ri) * geo.Hq + h + hh) * kD + c0;
 #pragma unroll
             for (int c4 = 0; c4 < 2; ++c4) {
                 uint32_t u[32];
                 ptx::tmem_ld32(tmem + kColO + c0 + c4 * 32 + lane_base, u);
                 ptx::tmem_wait_ld();
                 ptx::reg_fence(u);
-                if (r < rows) {
+                if (ri < rows && hh < hn) {
 #pragma unroll
                     for (int e = 0; e < 32; ++e) nf = fmaf(__uint_as_float(u[e]), 0.f, nf);
                     if (a.out_dtype == KL_FP32) {
@@ -625,6 +658,83 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (__any_sync(0xffffffffu, nf != nf) && lane == 0) raise_flag(a.err, KL_FLAG_RANGE);
         }
+    }
+
+    if (kShared && cs > 1) {
+        // Merge of the cluster's states (m, l, O) as kl_combine does: every CTA scales its O to the
+        // cluster's maximum and sum and puts it into its idle ring; then CTA k adds up rows
+        // 128 k / cs .. of all of them. Every thread takes part in every cluster barrier.
+        constexpr uint32_t kXRow = kD * 4 + 16;   // bytes of a row in the ring
+        const uint32_t xch = ptx::smem_addr(sm.tiles[0]);
+        ptx::cluster_sync();
+        if (warp < kComputeWarps) {
+            const uint32_t mla = ptx::smem_addr(&sm.ml[r]);
+            float2 v[8];
+            float M = -INFINITY;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k < cs) {
+                    v[k] = ptx::ld_cluster_v2(ptx::cluster_addr(mla, k));
+                    if (v[k].y > 0.f) M = fmaxf(M, v[k].x);
+                }
+            }
+            float z = 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (k < cs && v[k].y > 0.f) z += v[k].y * ptx::ex2(v[k].x - M);
+            const float2 own = sm.ml[r];
+            // an empty state adds zeros; a NaN sum makes NaN outputs, as in an undivided block
+            const bool none = n_sub == 0 || own.y == 0.f;
+            const float w = own.y > 0.f ? ptx::ex2(own.x - M) / z : own.y;
+            const int c0 = hf * 64;
+#pragma unroll
+            for (int c4 = 0; c4 < 2; ++c4) {
+                uint32_t u[32];
+                if (n_sub > 0) {
+                    ptx::tc_fence_after();
+                    ptx::tmem_ld32(tmem + kColO + c0 + c4 * 32 + ((uint32_t)(qd * 32) << 16), u);
+                    ptx::tmem_wait_ld();
+                    ptx::reg_fence(u);
+                }
+#pragma unroll
+                for (int e = 0; e < 32; ++e)
+                    u[e] = none ? 0u : __float_as_uint(__uint_as_float(u[e]) * w);
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    st_shared_v4(xch + r * kXRow + (c0 + c4 * 32 + 4 * c) * 4, u[4 * c], u[4 * c + 1],
+                                 u[4 * c + 2], u[4 * c + 3]);
+            }
+        }
+        ptx::cluster_sync();
+        if (warp < kComputeWarps) {
+            // one warp per row, 4 dims per lane
+            const int per = kBM / cs;
+            float nf = 0.f;
+            for (int i = warp; i < per; i += kComputeWarps) {
+                const int row = rank * per + i, ri = row / hp, hh = row - ri * hp;
+                if (ri >= rows || hh >= hn) continue;
+                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (k < cs) {
+                        const float4 x = ptx::ld_cluster_v4(ptx::cluster_addr(xch + row * kXRow + lane * 16, k));
+                        o.x += x.x;
+                        o.y += x.y;
+                        o.z += x.z;
+                        o.w += x.w;
+                    }
+                }
+                nf = fmaf(o.x, 0.f, fmaf(o.y, 0.f, fmaf(o.z, 0.f, fmaf(o.w, 0.f, nf))));
+                const size_t oi = ((size_t)(q0 + m0 + ri) * geo.Hq + h + hh) * kD + 4 * lane;
+                if (a.out_dtype == KL_FP32)
+                    *reinterpret_cast<float4 *>(static_cast<float *>(a.out) + oi) = o;
+                else
+                    *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(a.out) + oi) =
+                        make_uint2(pack2(o.x, o.y), pack2(o.z, o.w));
+            }
+            if (__any_sync(0xffffffffu, nf != nf) && lane == 0) raise_flag(a.err, KL_FLAG_RANGE);
+        }
+        ptx::cluster_sync();      // no CTA leaves while another reads its ring
     }
 
     ptx::tc_fence_before();
@@ -715,6 +825,26 @@ bool prefill_tc_supported(const Geometry &g) {
 cudaError_t launch_prefill_tc(const PrefillArgs &a) {
     const Geometry &g = a.geo;
     if (g.B == 0 || a.total_q == 0 || a.max_q == 0) return cudaSuccess;
+    PrefillArgs la = a;
+    // Heads per block: a block's 128 rows hold hp heads of a group (which read the same tiles),
+    // 128 / hp query rows each; the fewest blocks, and the fewest heads among equals. One W^R per
+    // query head: one head per block, which has one routing matrix.
+    auto blocks_of = [&](int hp) {
+        return (int64_t)((g.G + hp - 1) / hp) * ((a.max_q + kBM / hp - 1) / (kBM / hp));
+    };
+    if (!g.wr_per_qh)
+        for (int hp = 2; hp <= g.G && hp <= 64; ++hp)
+            if (blocks_of(hp) < blocks_of(la.hp)) la.hp = hp;
+    la.rpb = kBM / la.hp;
+    // CTAs per block: while the blocks leave half of the SMs idle, clusters of 2, 4 or 8 CTAs
+    // split a block's tiles (at least two tiles each at the longest length). A cluster's CTAs sit
+    // in one GPC, which leaves some of its SMs over: 15/16 of them are counted on for pairs, 27/32
+    // for clusters of 4 and 8.
+    const int64_t blocks = blocks_of(la.hp) * g.Hkv * g.B;
+    const int64_t tiles = ((int64_t)g.max_pages * g.P + kBN - 1) / kBN;
+    while (la.cs < 8 && la.cs * 4 <= tiles &&
+           blocks * la.cs * 2 * 32 <= (int64_t)device_sm_count() * (la.cs == 1 ? 30 : 27))
+        la.cs *= 2;
     CUtensorMap vmap, wmap, qmap;
     {
         // cache as [num_pages * Hkv * P rows][128], one box = one page of one head (64 dims)
@@ -732,27 +862,34 @@ cudaError_t launch_prefill_tc(const PrefillArgs &a) {
         if (!encode(&wmap, a.w_r, 2, dims, strides, box)) return cudaErrorInvalidValue;
     }
     {
-        // q as [total_q][Hq][128], one box = 128 consecutive rows of one head (64 dims); rows
-        // past total_q read as zeros
+        // q as [total_q][Hq][128], one box = rpb consecutive rows of hp heads (64 dims); rows past
+        // total_q and heads past Hq read as zeros
         const cuuint64_t dims[3] = {kD, (cuuint64_t)g.Hq, (cuuint64_t)a.total_q};
         const cuuint64_t strides[2] = {kD * 2, (cuuint64_t)g.Hq * kD * 2};
-        const cuuint32_t box[3] = {64, 1, kBM};
+        const cuuint32_t box[3] = {64, (cuuint32_t)la.hp, (cuuint32_t)la.rpb};
         if (!encode(&qmap, a.q, 3, dims, strides, box)) return cudaErrorInvalidValue;
     }
     const size_t smem = sizeof(PrefillSmem) + 1024;
-    static PerDeviceOnce once;
-    const cudaError_t e = once.run([&] {
-        return cudaFuncSetAttribute(prefill_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem);
+    const bool shared = la.hp > 1 || la.cs > 1;
+    const auto kernel = shared ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
+    static PerDeviceOnce once[2];
+    const cudaError_t e = once[shared].run([&] {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(g.Hq, g.B, (a.max_q + kBM - 1) / kBM);
+    cfg.gridDim = dim3(la.cs * g.Hkv * ((g.G + la.hp - 1) / la.hp), g.B, (a.max_q + la.rpb - 1) / la.rpb);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = a.stream;
-    const OverlapAttr overlap(cfg);
-    return cudaLaunchKernelEx(&cfg, prefill_tc_kernel, vmap, wmap, qmap, a);
+    cudaLaunchAttribute attr[2];
+    attr[0] = OverlapAttr(cfg).attr[0];
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)la.cs;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = la.cs > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, vmap, wmap, qmap, la);
 }
 
 cudaError_t launch_append_chunk(const Geometry &g, int total_q, int max_q, const uint16_t *v_new,
