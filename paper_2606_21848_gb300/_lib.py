@@ -115,31 +115,21 @@ def status_string(status: int) -> str:
         return "unknown"
 
 
-# A small decode takes the GPU 6 to 8 us, so the binding has to cost less than that per call:
-# addresses go to ctypes as plain ints (the argtypes convert them; a c_void_p object per argument
-# and the Stream object of torch.cuda.current_stream() took 17 us of host time per decode step
-# where this takes 5).
 def _p(x):
-    """The device address of a tensor, or the given address (an int or None)."""
-    if x is None or isinstance(x, int):
-        return x
-    return x.data_ptr()
-
-
-_torch = None
+    if x is None:
+        return None
+    if isinstance(x, int):
+        return ctypes.c_void_p(x)
+    return ctypes.c_void_p(x.data_ptr())
 
 
 def _stream(stream):
-    """The raw handle of a stream: a torch stream, an int, or None for torch's current stream."""
-    if stream is not None:
-        return stream if isinstance(stream, int) else stream.cuda_stream
-    global _torch
-    if _torch is None:
+    if stream is None:
         import torch
-        _torch = torch
-    if _torch.cuda.is_initialized():
-        return _torch._C._cuda_getCurrentRawStream(_torch._C._cuda_getDevice())
-    return _torch.cuda.current_stream().cuda_stream   # initializes CUDA
+        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if isinstance(stream, int):
+        return ctypes.c_void_p(stream)
+    return ctypes.c_void_p(stream.cuda_stream)
 
 
 def _nbytes(t) -> int:
