@@ -1,13 +1,17 @@
-"""ctypes binding of libkeyless (include/keyless.h): argument marshalling only.
+"""Binding of libkeyless (include/keyless.h): argument marshalling only.
 
 Every function has the C name and the C argument order; tensors are passed as torch CUDA
 tensors (or raw device addresses as ints) and the stream defaults to torch's current stream.
+The launching functions go through a small C module (csrc/kl_python.c), the others and the
+structures through ctypes.
 A non-OK status raises :class:`KLError`. There is no fallback: if the library has not been
 built, :func:`load` raises.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 import re
 
@@ -115,25 +119,21 @@ def status_string(status: int) -> str:
         return "unknown"
 
 
-def _p(x):
-    if x is None:
-        return None
-    if isinstance(x, int):
-        return ctypes.c_void_p(x)
-    return ctypes.c_void_p(x.data_ptr())
+_native = None
 
 
-def _stream(stream):
-    if stream is None:
-        import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
-
-
-def _nbytes(t) -> int:
-    return 0 if t is None else t.numel() * t.element_size()
+def _call():
+    """The marshalling module (csrc/kl_python.c), loaded next to the library."""
+    global _native
+    if _native is None:
+        load()
+        if not os.path.exists(_build.PYMOD):
+            raise RuntimeError(f"the binding is not built ({_build.PYMOD} missing); call build() first")
+        loader = importlib.machinery.ExtensionFileLoader("_keyless", _build.PYMOD)
+        spec = importlib.util.spec_from_file_location("_keyless", _build.PYMOD, loader=loader)
+        _native = importlib.util.module_from_spec(spec)
+        loader.exec_module(_native)
+    return _native
 
 
 def _check(status: int, where: str):
@@ -148,13 +148,12 @@ def make_shape(num_seqs, num_q_heads, num_kv_heads, head_dim, page_size, num_pag
 
 
 def kl_route_query(shape, q, w_r, q_r, stream=None):
-    _check(load().kl_route_query(ctypes.byref(shape), _p(q), _p(w_r), _p(q_r), _stream(stream)),
-           "kl_route_query")
+    _check(_call().kl_route_query(shape, q, w_r, q_r, stream), "kl_route_query")
 
 
 def kl_append_v(shape, v_new, block_table, positions, v_cache, err=None, stream=None):
-    _check(load().kl_append_v(ctypes.byref(shape), _p(v_new), _p(block_table), _p(positions),
-                              _p(v_cache), _p(err), _stream(stream)), "kl_append_v")
+    _check(_call().kl_append_v(shape, v_new, block_table, positions, v_cache, err, stream),
+           "kl_append_v")
 
 
 def kl_decode_workspace_size(shape, num_splits=0) -> int:
@@ -167,96 +166,81 @@ def kl_decode_num_splits(shape, num_splits=0) -> int:
 
 def kl_decode_attention(shape, q, w_r, v_cache, block_table, seq_lens, num_splits, out,
                         out_dtype, workspace, err=None, stream=None):
-    _check(load().kl_decode_attention(ctypes.byref(shape), _p(q), _p(w_r), _p(v_cache),
-                                      _p(block_table), _p(seq_lens), num_splits, _p(out),
-                                      out_dtype, _p(workspace), _nbytes(workspace), _p(err),
-                                      _stream(stream)), "kl_decode_attention")
+    _check(_call().kl_decode_attention(shape, q, w_r, v_cache, block_table, seq_lens, num_splits,
+                                       out, out_dtype, workspace, err, stream),
+           "kl_decode_attention")
 
 
 def kl_decode_attention_ex(shape, q, w_r, v_cache, block_table, seq_lens, opts, out,
                            out_dtype, workspace, err=None, stream=None):
-    _check(load().kl_decode_attention_ex(ctypes.byref(shape), _p(q), _p(w_r), _p(v_cache),
-                                         _p(block_table), _p(seq_lens),
-                                         None if opts is None else ctypes.byref(opts), _p(out),
-                                         out_dtype, _p(workspace), _nbytes(workspace), _p(err),
-                                         _stream(stream)), "kl_decode_attention_ex")
+    _check(_call().kl_decode_attention_ex(shape, q, w_r, v_cache, block_table, seq_lens, opts,
+                                          out, out_dtype, workspace, err, stream),
+           "kl_decode_attention_ex")
 
 
 def kl_decode_step(shape, q, w_r, v_new, positions, v_cache, block_table, seq_lens, opts, out,
                    out_dtype, workspace, err=None, stream=None):
     """Append of the current token's rows fused with the keyless decode (one pass)."""
-    _check(load().kl_decode_step(ctypes.byref(shape), _p(q), _p(w_r), _p(v_new), _p(positions),
-                                 _p(v_cache), _p(block_table), _p(seq_lens),
-                                 None if opts is None else ctypes.byref(opts), _p(out),
-                                 out_dtype, _p(workspace), _nbytes(workspace), _p(err),
-                                 _stream(stream)), "kl_decode_step")
+    _check(_call().kl_decode_step(shape, q, w_r, v_new, positions, v_cache, block_table, seq_lens,
+                                  opts, out, out_dtype, workspace, err, stream), "kl_decode_step")
 
 
 def kl_combine(shape, partial_o, partial_ml, num_splits, out, out_dtype, stream=None):
-    _check(load().kl_combine(ctypes.byref(shape), _p(partial_o), _p(partial_ml), num_splits,
-                             _p(out), out_dtype, _stream(stream)), "kl_combine")
+    _check(_call().kl_combine(shape, partial_o, partial_ml, num_splits, out, out_dtype, stream),
+           "kl_combine")
 
 
 def kl_standard_decode(shape, q, k_cache, v_cache, block_table, seq_lens, opts, out, out_dtype,
                        workspace, err=None, stream=None):
-    _check(load().kl_standard_decode(ctypes.byref(shape), _p(q), _p(k_cache), _p(v_cache),
-                                     _p(block_table), _p(seq_lens),
-                                     None if opts is None else ctypes.byref(opts), _p(out),
-                                     out_dtype, _p(workspace), _nbytes(workspace), _p(err),
-                                     _stream(stream)), "kl_standard_decode")
+    _check(_call().kl_standard_decode(shape, q, k_cache, v_cache, block_table, seq_lens, opts,
+                                      out, out_dtype, workspace, err, stream),
+           "kl_standard_decode")
 
 
 def kl_decode_attention_noalloc(shape, q, w_r, v_cache, block_table, seq_lens, num_splits, out,
                                 out_dtype, err=None, stream=None):
     """The decode with its split states in the library's fixed device scratch (no workspace)."""
-    _check(load().kl_decode_attention_noalloc(ctypes.byref(shape), _p(q), _p(w_r), _p(v_cache),
-                                              _p(block_table), _p(seq_lens), num_splits, _p(out),
-                                              out_dtype, _p(err), _stream(stream)),
+    _check(_call().kl_decode_attention_noalloc(shape, q, w_r, v_cache, block_table, seq_lens,
+                                               num_splits, out, out_dtype, err, stream),
            "kl_decode_attention_noalloc")
 
 
 def kl_append_v_chunk(shape, v_new, block_table, seq_lens, cu_q_lens, total_q, max_q_len, v_cache,
                       err=None, stream=None):
-    _check(load().kl_append_v_chunk(ctypes.byref(shape), _p(v_new), _p(block_table), _p(seq_lens),
-                                    _p(cu_q_lens), total_q, max_q_len, _p(v_cache), _p(err),
-                                    _stream(stream)), "kl_append_v_chunk")
+    _check(_call().kl_append_v_chunk(shape, v_new, block_table, seq_lens, cu_q_lens, total_q,
+                                     max_q_len, v_cache, err, stream), "kl_append_v_chunk")
 
 
 def kl_prefill_attention(shape, q, w_r, v_cache, block_table, seq_lens, cu_q_lens, total_q,
                          max_q_len, out, out_dtype, err=None, stream=None):
-    _check(load().kl_prefill_attention(ctypes.byref(shape), _p(q), _p(w_r), _p(v_cache),
-                                       _p(block_table), _p(seq_lens), _p(cu_q_lens), total_q,
-                                       max_q_len, _p(out), out_dtype, _p(err), _stream(stream)),
+    _check(_call().kl_prefill_attention(shape, q, w_r, v_cache, block_table, seq_lens, cu_q_lens,
+                                        total_q, max_q_len, out, out_dtype, err, stream),
            "kl_prefill_attention")
 
 
 def kl_append_v_fp8(shape, v_new, block_table, positions, v_codes, v_scales, err=None,
                     stream=None):
-    _check(load().kl_append_v_fp8(ctypes.byref(shape), _p(v_new), _p(block_table), _p(positions),
-                                  _p(v_codes), _p(v_scales), _p(err), _stream(stream)),
-           "kl_append_v_fp8")
+    _check(_call().kl_append_v_fp8(shape, v_new, block_table, positions, v_codes, v_scales, err,
+                                   stream), "kl_append_v_fp8")
 
 
 def kl_quantize_cache_fp8(shape, v_cache, v_codes, v_scales, stream=None):
-    _check(load().kl_quantize_cache_fp8(ctypes.byref(shape), _p(v_cache), _p(v_codes),
-                                        _p(v_scales), _stream(stream)), "kl_quantize_cache_fp8")
+    _check(_call().kl_quantize_cache_fp8(shape, v_cache, v_codes, v_scales, stream),
+           "kl_quantize_cache_fp8")
 
 
 def kl_decode_attention_fp8(shape, q, w_r, v_codes, v_scales, block_table, seq_lens, num_splits,
                             out, out_dtype, workspace, err=None, stream=None):
-    _check(load().kl_decode_attention_fp8(ctypes.byref(shape), _p(q), _p(w_r), _p(v_codes),
-                                          _p(v_scales), _p(block_table), _p(seq_lens), num_splits,
-                                          _p(out), out_dtype, _p(workspace), _nbytes(workspace),
-                                          _p(err), _stream(stream)), "kl_decode_attention_fp8")
+    _check(_call().kl_decode_attention_fp8(shape, q, w_r, v_codes, v_scales, block_table,
+                                           seq_lens, num_splits, out, out_dtype, workspace, err,
+                                           stream), "kl_decode_attention_fp8")
 
 
 def kl_decode_step_fp8(shape, q, w_r, v_new, positions, v_codes, v_scales, block_table, seq_lens,
                        num_splits, out, out_dtype, workspace, err=None, stream=None):
-    _check(load().kl_decode_step_fp8(ctypes.byref(shape), _p(q), _p(w_r), _p(v_new), _p(positions),
-                                     _p(v_codes), _p(v_scales), _p(block_table), _p(seq_lens),
-                                     num_splits, _p(out), out_dtype, _p(workspace),
-                                     _nbytes(workspace), _p(err), _stream(stream)),
-           "kl_decode_step_fp8")
+    _check(_call().kl_decode_step_fp8(shape, q, w_r, v_new, positions, v_codes, v_scales,
+                                      block_table, seq_lens, num_splits, out, out_dtype,
+                                      workspace, err, stream), "kl_decode_step_fp8")
 
 
 def make_latent_shape(num_seqs, num_q_heads, num_latent_heads, head_dim, latent_dim, page_size,
@@ -272,19 +256,16 @@ def kl_latent_workspace_size(shape, num_splits=0) -> int:
 
 def kl_latent_decode(shape, q, w_r, w_post, v_lat, block_table, seq_lens, num_splits, out,
                      out_dtype, workspace, err=None, stream=None):
-    _check(load().kl_latent_decode(ctypes.byref(shape), _p(q), _p(w_r), _p(w_post), _p(v_lat),
-                                   _p(block_table), _p(seq_lens), num_splits, _p(out), out_dtype,
-                                   _p(workspace), _nbytes(workspace), _p(err), _stream(stream)),
+    _check(_call().kl_latent_decode(shape, q, w_r, w_post, v_lat, block_table, seq_lens,
+                                    num_splits, out, out_dtype, workspace, err, stream),
            "kl_latent_decode")
 
 
 def kl_latent_decode_step(shape, q, w_r, w_post, v_new, positions, v_lat, block_table, seq_lens,
                           num_splits, out, out_dtype, workspace, err=None, stream=None):
-    _check(load().kl_latent_decode_step(ctypes.byref(shape), _p(q), _p(w_r), _p(w_post), _p(v_new),
-                                        _p(positions), _p(v_lat), _p(block_table), _p(seq_lens),
-                                        num_splits, _p(out), out_dtype, _p(workspace),
-                                        _nbytes(workspace), _p(err), _stream(stream)),
-           "kl_latent_decode_step")
+    _check(_call().kl_latent_decode_step(shape, q, w_r, w_post, v_new, positions, v_lat,
+                                         block_table, seq_lens, num_splits, out, out_dtype,
+                                         workspace, err, stream), "kl_latent_decode_step")
 
 
 def kl_decode_kernel_available(shape, kernel, standard=False) -> bool:

@@ -2,7 +2,8 @@
 
 Each translation unit under ``csrc/`` is compiled in parallel to an object file, then the
 objects are linked into ``_build/libkeyless.so`` with the CUDA runtime linked statically, so
-the library has no dependency beyond the driver. Rebuilds only when a source is newer than
+the library has no dependency beyond the driver; the binding's C module
+(``csrc/kl_python.c``) is compiled next to it. Rebuilds only when a source is newer than
 the library.
 """
 from __future__ import annotations
@@ -11,6 +12,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -19,6 +21,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libkeyless.so")
+PYSRC = os.path.join(CSRC, "kl_python.c")
+PYMOD = os.path.join(BUILD, "_keyless.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
@@ -37,10 +41,10 @@ def sources() -> list[str]:
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYMOD):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYMOD))
+    deps = sources() + [PYSRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(p) > t for p in deps)
 
 
@@ -70,6 +74,15 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | N
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
+    # the Python module beside it (host C, linked to the library in its own folder)
+    tmp = PYMOD + ".tmp"
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", INCLUDE,
+           "-I", sysconfig.get_paths()["include"], PYSRC, "-o", tmp, "-L", BUILD, "-l:libkeyless.so",
+           "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"building the Python module failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, PYMOD)
     return LIB
 
 

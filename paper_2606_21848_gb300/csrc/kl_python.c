@@ -1,0 +1,233 @@
+/*
+ * Argument marshalling of the Python binding (_lib.py) in C: one function per launching entry
+ * point of libkeyless. An address argument is None, an int, or an object with data_ptr(); a shape or
+ * options argument is the ctypes structure of _lib.py; the stream is None (torch's current
+ * stream), an int, or an object with cuda_stream. Each returns the kl_status.
+ *
+ * A small decode takes the GPU 6 to 8 us and the C call 2, while ctypes with a c_void_p object per
+ * argument and torch.cuda.current_stream() took 15 us of host time in front of it, plain ints and
+ * the raw stream through ctypes 6, and this takes about 2.
+ */
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <stdint.h>
+#include <string.h>
+
+#include "keyless.h"
+
+static PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream;
+static PyObject *g_argument_error;                        /* ctypes.ArgumentError */
+static PyObject *g_initialized, *g_get_device, *g_raw_stream, *g_current_stream;   /* torch */
+
+static int to_u64(PyObject *v, uint64_t *out) {
+    *out = PyLong_AsUnsignedLongLongMask(v);
+    return !(*out == (uint64_t)-1 && PyErr_Occurred());
+}
+
+static int get_addr(PyObject *o, void **out) {
+    uint64_t x = 0;
+    if (o == Py_None) {
+        *out = NULL;
+        return 1;
+    }
+    if (PyLong_Check(o)) {
+        if (!to_u64(o, &x)) return 0;
+    } else {
+        PyObject *v = PyObject_CallMethodNoArgs(o, s_data_ptr);
+        if (!v) return 0;
+        const int ok = to_u64(v, &x);
+        Py_DECREF(v);
+        if (!ok) return 0;
+    }
+    *out = (void *)(uintptr_t)x;
+    return 1;
+}
+
+static int get_i32(PyObject *o, int32_t *out) {
+    if (!PyLong_Check(o)) {
+        PyErr_Format(g_argument_error, "expected an int, got %.100s", Py_TYPE(o)->tp_name);
+        return 0;
+    }
+    const unsigned long v = PyLong_AsUnsignedLongMask(o);
+    if (v == (unsigned long)-1 && PyErr_Occurred()) return 0;
+    *out = (int32_t)v;
+    return 1;
+}
+
+/* The contents of a ctypes structure of exactly `size` bytes. */
+static int get_struct(PyObject *o, void *out, Py_ssize_t size) {
+    Py_buffer b;
+    if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) < 0) return 0;
+    const int ok = b.len == size;
+    if (ok) memcpy(out, b.buf, (size_t)size);
+    PyBuffer_Release(&b);
+    if (!ok) PyErr_SetString(g_argument_error, "a structure of another type");
+    return ok;
+}
+
+/* numel() * element_size() of a tensor, 0 of None. */
+static int get_nbytes(PyObject *o, size_t *out) {
+    uint64_t n, e;
+    if (o == Py_None) {
+        *out = 0;
+        return 1;
+    }
+    PyObject *v = PyObject_CallMethodNoArgs(o, s_numel);
+    if (!v) return 0;
+    int ok = to_u64(v, &n);
+    Py_DECREF(v);
+    if (!ok) return 0;
+    v = PyObject_CallMethodNoArgs(o, s_element_size);
+    if (!v) return 0;
+    ok = to_u64(v, &e);
+    Py_DECREF(v);
+    *out = (size_t)(n * e);
+    return ok;
+}
+
+static int find_torch(void) {
+    PyObject *cuda = PyImport_ImportModule("torch.cuda"), *c = PyImport_ImportModule("torch._C");
+    int ok = cuda && c;
+    ok = ok && (g_current_stream = PyObject_GetAttrString(cuda, "current_stream"));
+    ok = ok && (g_get_device = PyObject_GetAttrString(c, "_cuda_getDevice"));
+    ok = ok && (g_raw_stream = PyObject_GetAttrString(c, "_cuda_getCurrentRawStream"));
+    ok = ok && (g_initialized = PyObject_GetAttrString(cuda, "is_initialized"));   /* last: the mark */
+    Py_XDECREF(cuda);
+    Py_XDECREF(c);
+    return ok;
+}
+
+static int get_stream(PyObject *o, kl_stream_t *out) {
+    uint64_t x = 0;
+    PyObject *v;
+    if (PyLong_Check(o)) {
+        if (!to_u64(o, &x)) return 0;
+    } else if (o != Py_None) {
+        v = PyObject_GetAttr(o, s_cuda_stream);
+        if (!v) return 0;
+        const int ok = to_u64(v, &x);
+        Py_DECREF(v);
+        if (!ok) return 0;
+    } else {
+        if (!g_initialized && !find_torch()) return 0;
+        v = PyObject_CallNoArgs(g_initialized);
+        if (!v) return 0;
+        const int init = PyObject_IsTrue(v);
+        Py_DECREF(v);
+        if (init < 0) return 0;
+        if (!init) {                       /* current_stream() initializes CUDA */
+            v = PyObject_CallNoArgs(g_current_stream);
+            if (!v) return 0;
+            const int ok = get_stream(v, out);
+            Py_DECREF(v);
+            return ok;
+        }
+        PyObject *d = PyObject_CallNoArgs(g_get_device);
+        if (!d) return 0;
+        v = PyObject_CallOneArg(g_raw_stream, d);
+        Py_DECREF(d);
+        if (!v) return 0;
+        const int ok = to_u64(v, &x);
+        Py_DECREF(v);
+        if (!ok) return 0;
+    }
+    *out = (kl_stream_t)(uintptr_t)x;
+    return 1;
+}
+
+#define SHAPE(i) kl_shape sh; if (!get_struct(a[i], &sh, sizeof sh)) return NULL
+#define LATENT(i) kl_latent_shape sh; if (!get_struct(a[i], &sh, sizeof sh)) return NULL
+#define PTR(i, x) void *x; if (!get_addr(a[i], &x)) return NULL
+#define INT(i, x) int32_t x; if (!get_i32(a[i], &x)) return NULL
+#define OPTS(i) kl_decode_options o; const int has_o = a[i] != Py_None; \
+    if (has_o && !get_struct(a[i], &o, sizeof o)) return NULL
+#define WORK(i) void *ws; size_t wsn; if (!get_addr(a[i], &ws) || !get_nbytes(a[i], &wsn)) return NULL
+#define STREAM(i) kl_stream_t st; if (!get_stream(a[i], &st)) return NULL
+#define FN(name, n) static PyObject *py_##name(PyObject *m, PyObject *const *a, Py_ssize_t na) { \
+    (void)m; \
+    if (na != (n)) { PyErr_Format(PyExc_TypeError, #name " takes %d arguments", (n)); return NULL; }
+#define CALL(expr) kl_status r; Py_BEGIN_ALLOW_THREADS r = (expr); Py_END_ALLOW_THREADS \
+    return PyLong_FromLong((long)r); }
+
+FN(route_query, 5) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, out); STREAM(4);
+CALL(kl_route_query(&sh, q, w, out, st))
+
+FN(append_v, 7) SHAPE(0); PTR(1, v); PTR(2, bt); PTR(3, pos); PTR(4, c); PTR(5, e); STREAM(6);
+CALL(kl_append_v(&sh, v, bt, pos, c, e, st))
+
+FN(decode_attention, 12) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl); INT(6, ns);
+PTR(7, out); INT(8, dt); WORK(9); PTR(10, e); STREAM(11);
+CALL(kl_decode_attention(&sh, q, w, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(decode_attention_ex, 12) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl); OPTS(6);
+PTR(7, out); INT(8, dt); WORK(9); PTR(10, e); STREAM(11);
+CALL(kl_decode_attention_ex(&sh, q, w, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(decode_step, 14) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, v); PTR(4, pos); PTR(5, c); PTR(6, bt);
+PTR(7, sl); OPTS(8); PTR(9, out); INT(10, dt); WORK(11); PTR(12, e); STREAM(13);
+CALL(kl_decode_step(&sh, q, w, v, pos, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(combine, 7) SHAPE(0); PTR(1, po); PTR(2, ml); INT(3, ns); PTR(4, out); INT(5, dt); STREAM(6);
+CALL(kl_combine(&sh, po, ml, ns, out, (kl_dtype)dt, st))
+
+FN(standard_decode, 12) SHAPE(0); PTR(1, q); PTR(2, k); PTR(3, c); PTR(4, bt); PTR(5, sl); OPTS(6);
+PTR(7, out); INT(8, dt); WORK(9); PTR(10, e); STREAM(11);
+CALL(kl_standard_decode(&sh, q, k, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(decode_attention_noalloc, 11) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl);
+INT(6, ns); PTR(7, out); INT(8, dt); PTR(9, e); STREAM(10);
+CALL(kl_decode_attention_noalloc(&sh, q, w, c, bt, sl, ns, out, (kl_dtype)dt, e, st))
+
+FN(append_v_chunk, 10) SHAPE(0); PTR(1, v); PTR(2, bt); PTR(3, sl); PTR(4, cu); INT(5, tq); INT(6, mq);
+PTR(7, c); PTR(8, e); STREAM(9);
+CALL(kl_append_v_chunk(&sh, v, bt, sl, cu, tq, mq, c, e, st))
+
+FN(prefill_attention, 13) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl); PTR(6, cu);
+INT(7, tq); INT(8, mq); PTR(9, out); INT(10, dt); PTR(11, e); STREAM(12);
+CALL(kl_prefill_attention(&sh, q, w, c, bt, sl, cu, tq, mq, out, (kl_dtype)dt, e, st))
+
+FN(append_v_fp8, 8) SHAPE(0); PTR(1, v); PTR(2, bt); PTR(3, pos); PTR(4, c); PTR(5, s); PTR(6, e);
+STREAM(7);
+CALL(kl_append_v_fp8(&sh, v, bt, pos, c, s, e, st))
+
+FN(quantize_cache_fp8, 5) SHAPE(0); PTR(1, v); PTR(2, c); PTR(3, s); STREAM(4);
+CALL(kl_quantize_cache_fp8(&sh, v, c, s, st))
+
+FN(decode_attention_fp8, 13) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, s); PTR(5, bt); PTR(6, sl);
+INT(7, ns); PTR(8, out); INT(9, dt); WORK(10); PTR(11, e); STREAM(12);
+CALL(kl_decode_attention_fp8(&sh, q, w, c, s, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(decode_step_fp8, 15) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, v); PTR(4, pos); PTR(5, c); PTR(6, s);
+PTR(7, bt); PTR(8, sl); INT(9, ns); PTR(10, out); INT(11, dt); WORK(12); PTR(13, e); STREAM(14);
+CALL(kl_decode_step_fp8(&sh, q, w, v, pos, c, s, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(latent_decode, 13) LATENT(0); PTR(1, q); PTR(2, w); PTR(3, wp); PTR(4, c); PTR(5, bt); PTR(6, sl);
+INT(7, ns); PTR(8, out); INT(9, dt); WORK(10); PTR(11, e); STREAM(12);
+CALL(kl_latent_decode(&sh, q, w, wp, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+
+FN(latent_decode_step, 15) LATENT(0); PTR(1, q); PTR(2, w); PTR(3, wp); PTR(4, v); PTR(5, pos); PTR(6, c);
+PTR(7, bt); PTR(8, sl); INT(9, ns); PTR(10, out); INT(11, dt); WORK(12); PTR(13, e); STREAM(14);
+CALL(kl_latent_decode_step(&sh, q, w, wp, v, pos, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+
+#define M(name) {"kl_" #name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL}
+static PyMethodDef methods[] = {
+    M(route_query), M(append_v), M(decode_attention), M(decode_attention_ex), M(decode_step), M(combine),
+    M(standard_decode), M(decode_attention_noalloc), M(append_v_chunk), M(prefill_attention),
+    M(append_v_fp8), M(quantize_cache_fp8), M(decode_attention_fp8), M(decode_step_fp8),
+    M(latent_decode), M(latent_decode_step), {NULL, NULL, 0, NULL}};
+static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_keyless", NULL, -1, methods,
+                                    NULL, NULL, NULL, NULL};
+
+PyMODINIT_FUNC PyInit__keyless(void) {
+    PyObject *c = PyImport_ImportModule("ctypes");
+    if (!c) return NULL;
+    g_argument_error = PyObject_GetAttrString(c, "ArgumentError");
+    Py_DECREF(c);
+    if (!g_argument_error) return NULL;
+    if (!(s_data_ptr = PyUnicode_InternFromString("data_ptr")) ||
+        !(s_numel = PyUnicode_InternFromString("numel")) ||
+        !(s_element_size = PyUnicode_InternFromString("element_size")) ||
+        !(s_cuda_stream = PyUnicode_InternFromString("cuda_stream")))
+        return NULL;
+    return PyModule_Create(&module);
+}
