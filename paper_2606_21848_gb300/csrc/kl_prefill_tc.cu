@@ -871,26 +871,32 @@ cudaError_t launch_prefill_tc(const PrefillArgs &a) {
         if (!encode(&qmap, a.q, 3, dims, strides, box)) return cudaErrorInvalidValue;
     }
     const size_t smem = sizeof(PrefillSmem) + 1024;
-    const bool shared = la.hp > 1 || la.cs > 1;
-    const auto kernel = shared ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
-    static PerDeviceOnce once[2];
-    const cudaError_t e = once[shared].run([&] {
-        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    });
-    if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(la.cs * g.Hkv * ((g.G + la.hp - 1) / la.hp), g.B, (a.max_q + la.rpb - 1) / la.rpb);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = a.stream;
-    cudaLaunchAttribute attr[2];
-    attr[0] = OverlapAttr(cfg).attr[0];
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)la.cs;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = la.cs > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, vmap, wmap, qmap, la);
+    while (true) {
+        const bool shared = la.hp > 1 || la.cs > 1;
+        const auto kernel = shared ? prefill_tc_kernel<true> : prefill_tc_kernel<false>;
+        static PerDeviceOnce once[2];
+        cudaError_t e = once[shared].run([&] {
+            return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        });
+        if (e != cudaSuccess) return e;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(la.cs * g.Hkv * ((g.G + la.hp - 1) / la.hp), g.B, (a.max_q + la.rpb - 1) / la.rpb);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = a.stream;
+        cudaLaunchAttribute attr[2];
+        attr[0] = OverlapAttr(cfg).attr[0];
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)la.cs;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = la.cs > 1 ? 2 : 1;
+        e = cudaLaunchKernelEx(&cfg, kernel, vmap, wmap, qmap, la);
+        if (e == cudaSuccess || la.cs == 1) return e;
+        // a context that may not use enough SMs of one GPC for the cluster: one CTA per block
+        (void)cudaGetLastError();
+        la.cs = 1;
+    }
 }
 
 cudaError_t launch_append_chunk(const Geometry &g, int total_q, int max_q, const uint16_t *v_new,
