@@ -1,9 +1,9 @@
 """GB300-native decode (and chunked prefill) of Keyless Attention over a paged Value-Only Cache.
 
 The compute lives in ``libkeyless.so`` (hand-written CUDA for sm_103a behind the C ABI of
-``include/keyless.h``); this package holds its build script, a ctypes binding with the same
-function names, and the seeded input generators. PyTorch is used for device memory and
-streams only.
+``include/keyless.h``); this package holds its build script, a binding (a small C module and
+ctypes) with the same function names, and the seeded input generators. PyTorch is used for
+device memory and streams only.
 """
 from .builder import build  # noqa: F401
 from ._lib import (  # noqa: F401

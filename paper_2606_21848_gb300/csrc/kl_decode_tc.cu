@@ -1,7 +1,7 @@
 // Tensor-core split-sequence decode: the host-side plan (tensor maps, splits per CTA, heads per
 // compute warp) and the head-dim-128 kernels of groups of up to 8 heads; the kernel itself is in
 // kl_decode_tc_kernel.cuh, the head-dim-64 kernels in kl_decode_tc64.cu, those of larger groups
-// in kl_decode_tc_groups.cu.
+// in kl_decode_wide.cu and kl_decode_tc_groups.cu.
 #include "kl_decode_tc_kernel.cuh"
 
 namespace kl {
@@ -17,8 +17,9 @@ cudaError_t launch_waits(const DecodeArgs &la, bool per_split, const CUtensorMap
 
 template <bool kStandard>
 cudaError_t launch(const DecodeArgs &a) {
-    // groups of more than 8 heads: one wide CTA per SM, unless the caller takes the split states
-    // (one per split) or the K+V comparison is asked for
+    // groups of more than 8 heads: wide CTAs of up to 32 heads, unless the caller takes the split
+    // states (one per split) or the K+V comparison is asked for (64 sequences of 128/8 heads, 8192
+    // tokens: 252 us with sibling CTAs, 163 wide; 256 of 32/1 heads: 248 and 105)
     if (!kStandard && a.geo.nhb > 1 && a.geo.D == 128 && (a.direct_out || a.merge_inside))
         return launch_tc_wide(a);
     DecodeArgs la = a;

@@ -1,6 +1,8 @@
 // Head-dim-128 instances of the tensor-core decode for the sibling CTAs of groups of more than
 // 8 query heads (4 heads on each of eight compute warps; the kernel is in
 // kl_decode_tc_kernel.cuh): compiled in their own translation unit, in parallel with the others.
+// They serve what kl_decode_wide.cu does not: split states for the caller, the K+V comparison and
+// split counts above the in-kernel merge's.
 #include "kl_decode_tc_kernel.cuh"
 
 namespace kl {

@@ -2,8 +2,9 @@
 // tcgen05 MMAs with TMEM accumulators, warp-specialized roles.
 //
 // One CTA per (run of splits, value head g, sequence b, block of up to 8 of the group's query
-// heads: groups of more than 8 heads run ceil(G / 8) sibling CTAs that read the same pages);
-// head_dim 128 or 64. The value-space routing (Section 2.2: q_r = q W^R) runs first, as tensor-core MMAs on
+// heads); head_dim 128 or 64. Groups of more than 8 heads go to kl_decode_wide.cu; where that
+// kernel does not serve them (split states for the caller, the K+V comparison, head dim 64, more
+// splits than the in-kernel merge takes) ceil(G / 8) sibling CTAs here read the same pages. The value-space routing (Section 2.2: q_r = q W^R) runs first, as tensor-core MMAs on
 // W^R tiles that stream through the ring, into a split-bf16 operand (q_r * scale * log2 e =
 // hi + lo, both bf16) for the G heads of the group.
 // Then each 128-token tile of cached value rows V_t [128 x 128] (Section 3) is used twice by
@@ -38,8 +39,7 @@
 //
 // This header holds the kernel template and its launch for one head dim; kl_decode_tc.cu
 // instantiates head dim 128 and the host-side plan, kl_decode_tc64.cu head dim 64 and
-// kl_decode_tc_groups.cu the CTAs of groups of more than 8 heads, so that they compile in
-// parallel.
+// kl_decode_tc_groups.cu the sibling CTAs, so that they compile in parallel.
 #pragma once
 
 #include <cudaTypedefs.h>
