@@ -820,25 +820,33 @@ cudaError_t launch_tc_wide(const DecodeArgs &a) {
     DecodeArgs la = a;
     Geometry &g = la.geo;
     const int64_t sms = device_sm_count();
-    // 32 heads per CTA read each tile once for a group of 17 or more; with fewer such CTAs than
-    // SMs, blocks of 16 spread the group over twice as many.
-    const int64_t units8 = (int64_t)g.B * g.Hkv;
-    const bool w32 = g.G > 16 && units8 * ((g.G + 31) / 32) * g.S >= sms;
+    // consecutive splits per CTA: the fewest that fit one wave (when the units alone do not fill
+    // it), and at most kWideMaxRuns states to merge
+    const auto splits_per_cta = [&](int64_t units, int64_t slots) {
+        int spc = (g.S + kWideMaxRuns - 1) / kWideMaxRuns;
+        if (g.S > 1 && units < slots)
+            while ((int64_t)((g.S + spc - 1) / spc) * units > slots) ++spc;
+        return spc;
+    };
+    // Groups of 17 or more heads: CTAs of 32 heads (1180 cycles per tile where HBM does not set the
+    // pace), unless CTAs of 16 (1010) have an SM each and not 6/5 as many splits to run.
+    // (Group of 32, measured with CTAs of 16 and of 32: 104 sequences of 8192 tokens 65.8 and 50.8 us,
+    // 77 64.7 and 49.0, 30 of 32768 in 4 splits 71.4 and 55.3, 150 of 1000 in a group of 24 14.8 and
+    // 13.6; 52 sequences of 8192, one CTA of 16 on each of 104 SMs, 38.5 and about 45.)
+    const int64_t seq_heads = (int64_t)g.B * g.Hkv;
+    const int64_t units32 = seq_heads * ((g.G + 31) / 32), units16 = seq_heads * ((g.G + 15) / 16);
+    const bool w32 = g.G > 16 && (units16 > sms || 6 * splits_per_cta(units32, sms) <=
+                                                       5 * splits_per_cta(units16, sms));
     const int NH = w32 ? 32 : 16;
     g.nhb = (g.G + NH - 1) / NH;
     g.qbox = g.G < NH ? g.G : NH;
     // Blocks of 16 heads that overflow one CTA per SM go two to an SM with one softmax group each:
     // their waves overlap, and the last one shares HBM evenly. (Within one wave, the
     // deeper ring and the two groups of a CTA that has its SM alone are faster.)
-    const int64_t units = units8 * g.nhb;
+    const int64_t units = w32 ? units32 : units16;
     const bool two_per_sm = !w32 && units > sms;
     const int64_t slots = two_per_sm ? 2 * sms : sms;
-    // consecutive splits per CTA: the fewest that fit one wave (when the units alone do not fill
-    // it), and at most kWideMaxRuns states to merge
-    int spc = (g.S + kWideMaxRuns - 1) / kWideMaxRuns;
-    if (g.S > 1 && units < slots)
-        while ((int64_t)((g.S + spc - 1) / spc) * units > slots) ++spc;
-    g.spc = spc;
+    g.spc = splits_per_cta(units, slots);
     CUtensorMap vmap, wmap, qmap;
     if (!make_map(&vmap, a.v_cache, kD, (uint64_t)g.num_pages * g.Hkv * g.P, (uint32_t)g.P))
         return cudaErrorInvalidValue;

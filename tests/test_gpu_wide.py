@@ -62,3 +62,16 @@ def test_runs_merged(G, splits):
     out, err = decode(to_dev(x), shape_of(x), num_splits=splits, out_dtype=kl.KL_BF16)
     assert err == 0
     assert_parity(out.float().cpu().numpy(), oracle_decode(x, _gpu.default_scale(x)), f"S {splits}")
+
+
+# CTAs of 32 heads that leave SMs idle: CTAs of 16 would share SMs (the first three) or run more
+# splits each (the last two)
+@pytest.mark.parametrize("B, Hkv, G, P, splits", [(77, 1, 32, 16, 1), (60, 1, 40, 16, 1),
+                                                  (151, 1, 17, 64, 1), (30, 1, 32, 16, 4),
+                                                  (19, 2, 24, 32, 3)])
+def test_partly_filled_wave(B, Hkv, G, P, splits):
+    lens = (EDGES * 8)[:B]
+    x = tiny(B=B, Hq=Hkv * G, Hkv=Hkv, D=128, P=P, lens=lens, seed=90 + G)
+    out, err = decode(to_dev(x), shape_of(x), num_splits=splits)
+    assert err == 0
+    assert_parity(out.cpu().numpy(), oracle_decode(x, _gpu.default_scale(x)), f"{B} {G} S {splits}")
