@@ -566,9 +566,11 @@ __global__ void __launch_bounds__(kThreads, 2)
             ok = ptx::bar_and(kBarGroup + grp, kGroupThreads, wait(&sm.r_full, 0));
             if (ok) {
                 ptx::tc_fence_after();
+                float rv[kNR];
+                ptx::tmem_ld16(tmem + kColR + lane_base, rv);
 #pragma unroll
                 for (int e = 0; e < KR; ++e)
-                    if (h1 + e < G) acc[e] = ptx::tmem_ld1(tmem + kColR + h1 + e + lane_base);
+                    if (h1 + e < G) acc[e] = grp ? rv[KR + e] : rv[e];
                 ptx::tc_fence_before();
             }
         } else {
@@ -806,11 +808,11 @@ __global__ void __launch_bounds__(kThreads, 2)
         // without a tile has an empty one)
         ok = ok && carried;
         const int mine = (n_tiles + 1 - grp) >> 1;                 // the group's tiles
-        if (ok && mine > 0) ok = wait(&sm.o_full[grp], (mine - 1) & 1);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1)
 #pragma unroll
             for (int h = 0; h < Sh::NH; ++h) lsum[h] += __shfl_xor_sync(0xffffffffu, lsum[h], off);
+        if (ok && mine > 0) ok = wait(&sm.o_full[grp], (mine - 1) & 1);
         // (the barrier ahead keeps these writes behind the last slow tile's reads of red)
         ptx::bar_sync(kBarGroup + grp, kGroupThreads);
         if (lane == 0) {
@@ -821,11 +823,17 @@ __global__ void __launch_bounds__(kThreads, 2)
         if (ptx::bar_and(kBarComputeAnd, kComputeThreads, ok)) {
             ptx::tc_fence_after();
             const bool two = n_tiles > 1;
-            // O = (O_0 + O_1 / 16 + O_2 / 256) * inv of head h of a group
-            auto group_o = [&](int gi, int h) {
-                const uint32_t oc = tmem + kColO + 32 * gi + 16 * (h >> 2) + (h & 3) + lane_base;
-                const float o0 = ptx::tmem_ld1(oc), o1 = ptx::tmem_ld1(oc + 4), o2 = ptx::tmem_ld1(oc + 8);
-                return fmaf(o2, 1.f / 256.f, fmaf(o1, 1.f / 16.f, o0)) * sm.winv[gi];
+            // O = (O_0 + O_1 / 16 + O_2 / 256) * inv of head h1 + e of a group; the block's columns
+            // in one load (a load and a wait per term and head were 0.3 us of a CTA's end: 173
+            // sequences of 300 tokens, 64/8 heads, 51.0 -> 47.4 us with it, one load per warp for the
+            // routed query and the sums reduced before the wait on the last output MMAs)
+            float ov0[16], ov1[16];
+            const uint32_t oc = tmem + kColO + 16 * (h1 >> 2) + lane_base;
+            ptx::tmem_ld16(oc, ov0);
+            if (two) ptx::tmem_ld16(oc + 32, ov1);
+            auto group_o = [&](const float (&ov)[16], int gi, int e) {
+                auto term = [&](int j) { return NB == 1 && grp ? ov[4 * j + KR + e] : ov[4 * j + e]; };
+                return fmaf(term(2), 1.f / 256.f, fmaf(term(1), 1.f / 16.f, term(0))) * sm.winv[gi];
             };
 #pragma unroll
             for (int e = 0; e < KR; ++e) {
@@ -835,10 +843,10 @@ __global__ void __launch_bounds__(kThreads, 2)
                 const float M = fmaxf(m0, m1);
                 const float w0 = ptx::ex2(m0 - M), w1 = two ? ptx::ex2(m1 - M) : 0.f;
                 float lt = w0 * ((sm.red[0][0][h] + sm.red[0][1][h]) + (sm.red[0][2][h] + sm.red[0][3][h]));
-                float o = w0 * group_o(0, h);
+                float o = w0 * group_o(ov0, 0, e);
                 if (two) {
                     lt += w1 * ((sm.red[1][0][h] + sm.red[1][1][h]) + (sm.red[1][2][h] + sm.red[1][3][h]));
-                    o += w1 * group_o(1, h);
+                    o += w1 * group_o(ov1, 1, e);
                 }
                 const float val = o / lt;
                 const size_t bh = (size_t)b * geo.Hq + qh0 + h;
