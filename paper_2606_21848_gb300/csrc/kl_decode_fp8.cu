@@ -25,7 +25,7 @@
 // addresses. So the eight compute warps form two groups of four that take alternate tiles, each
 // thread with all (8 or 4) heads of its token, and each group with its own softmax state and O,
 // merged at the end like two splits. With all eight warps on every tile, half the heads each, the
-// 70B batch (256 x 64/8 heads, 8192 tokens) ran 437 us, now 370 us (the HBM floor is 327);
+// 70B batch (256 x 64/8 heads, 8192 tokens) ran 437 us, now 359 us (the HBM floor is 327);
 // 64 ragged sequences of 32/8 heads 254 -> 204 us, together with the one-lane page loop.
 //
 // The softmax keeps a lazy reference maximum per head: a tile's weights are 2^(s - m) with the
