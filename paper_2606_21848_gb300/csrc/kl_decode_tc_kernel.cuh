@@ -616,6 +616,9 @@ __global__ void __launch_bounds__(Roles<KH>::kThreads, 2)
     // of a zero-length sequence writes the zero output, and the empty splits of a longer
     // sequence take no part (the merge counts only the splits that hold tokens).
     if (n_tiles == 0) {
+        // (the latent decode: if every sequence is empty, nothing else holds this grid, and with it
+        // the kernels behind it, back until the absorbed-query kernel has finished its stores)
+        if (a.pdl) grid_dep_wait();
         if (app_owner && warp < geo.vpc) {
             const int page = bt[pos_raw / geo.P];
             const int gv = g + warp;                  // one warp per value head of the CTA

@@ -72,7 +72,7 @@ struct DecodeArgs {
     // Latent path, behind the absorbed-query kernel (which signals once everything ahead of it in
     // the stream has completed): the CTAs set up and fill their ring of cache tiles at once,
     // every role then sleeps in grid_dep_wait until that kernel has finished (the compute warps
-    // before reading q_routed).
+    // before reading q_routed; a CTA with an empty run before it ends).
     bool pdl = false;
 };
 
@@ -116,15 +116,25 @@ __device__ __forceinline__ void grid_dep_launch() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Launch attribute of every kernel here: a programmatic dependent of the kernel ahead of it in the
-// stream. Where that kernel signals early (these kernels but the prefill do, once all of their
-// CTAs run), the launch latency and the set-up overlap its end; each kernel calls grid_dep_wait()
-// in all threads before its first access to global memory (through pointers without __restrict__,
-// whose loads the compiler may not move above the wait), so stream order holds for everything it
-// reads and writes, and signals only once it holds its tensor memory, so that no CTA that waits
-// for it can take that. Behind any other kernel it starts as an ordinary launch. Calls one after
-// another: 8 x 4096 tokens 20.0 -> 16.9 us, one sequence of 131072 49.4 -> 47.0 us, 32 x 8192 at
-// head dim 64 86.2 -> 81.9 us, the 70B batch 604 -> 594 us.
+// Launch attribute of a programmatic dependent of the kernel ahead of it in the stream: of every
+// kernel here but the CUDA-core decode, route_kernel and quantize_rows_kernel (ordinary launches).
+// Where the kernel ahead signals early (all of these but the prefill and the latent expansion do,
+// once all of their CTAs run), the launch latency and the set-up overlap its end; behind any other
+// kernel it starts as an ordinary launch.
+//
+// Stream order holds because each kernel calls grid_dep_wait() in all threads before its first
+// access to global memory (through pointers without __restrict__, whose loads the compiler may not
+// move above the wait). The two kernels behind the latent path's absorbed-query kernel start
+// earlier: the decode reads lengths, table and cache and appends, and the expansion reads W_post,
+// before they wait. The absorbed-query kernel signals only after its own wait, so all that was
+// ahead of the call has completed by then; every CTA of the decode, one with an empty run too,
+// then waits for the absorbed-query kernel, and the expansion (one lane, before it reads the
+// decode's output; no CTA ends without it) for the decode, so that what waits for the expansion
+// waits for all three.
+//
+// A kernel signals only once it holds its tensor memory, so that no CTA that waits for it can take
+// that. Calls one after another: 8 x 4096 tokens 20.0 -> 16.9 us, one sequence of 131072
+// 49.4 -> 47.0 us, 32 x 8192 at head dim 64 86.2 -> 81.9 us, the 70B batch 604 -> 594 us.
 struct OverlapAttr {
     cudaLaunchAttribute attr[1];
     explicit OverlapAttr(cudaLaunchConfig_t &cfg) {
