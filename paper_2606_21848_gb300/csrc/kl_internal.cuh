@@ -83,7 +83,7 @@ struct PrefillArgs {
     Geometry geo;             // S and chunk unused
     int total_q;              // rows of q and out
     int max_q;                // host bound on n_b (grid sizing)
-    // Layout (set by the launcher): a block of 128 rows holds hp heads of one value head's group,
+    // Layout (set by the launcher, plan_prefill): a block of 128 rows holds hp heads of one value head's group,
     // rpb query rows each; a cluster of cs CTAs splits a block's cache tiles.
     int hp = 1, rpb = 128, cs = 1;
     const uint16_t *q;        // [total_q][Hq][D] bf16

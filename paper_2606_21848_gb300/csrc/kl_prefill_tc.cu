@@ -64,14 +64,15 @@
 #include <math.h>
 
 #include "kl_internal.cuh"
+#include "kl_prefill_plan.cuh"
 #include "kl_tc_ptx.cuh"
 
 namespace kl {
 namespace {
 
 constexpr int kD = 128;
-constexpr int kBM = 128;                          // query rows per CTA
-constexpr int kBN = 128;                          // cache rows per tile
+constexpr int kBM = kPrefillRows;                 // query rows per CTA
+constexpr int kBN = kPrefillTile;                 // cache rows per tile
 constexpr int kBS = 64;                           // cache rows per half tile
 constexpr int kSub = 4;                           // half tiles in flight (score buffers)
 constexpr int kStages = 5;
@@ -826,26 +827,11 @@ cudaError_t launch_prefill_tc(const PrefillArgs &a) {
     const Geometry &g = a.geo;
     if (g.B == 0 || a.total_q == 0 || a.max_q == 0) return cudaSuccess;
     PrefillArgs la = a;
-    // Heads per block: a block's 128 rows hold hp heads of a group (which read the same tiles),
-    // 128 / hp query rows each; the fewest blocks, and the fewest heads among equals. One W^R per
-    // query head: one head per block, which has one routing matrix.
-    auto blocks_of = [&](int hp) {
-        return (int64_t)((g.G + hp - 1) / hp) * ((a.max_q + kBM / hp - 1) / (kBM / hp));
-    };
-    if (!g.wr_per_qh)
-        for (int hp = 2; hp <= g.G && hp <= 64; ++hp)
-            if (blocks_of(hp) < blocks_of(la.hp)) la.hp = hp;
-    la.rpb = kBM / la.hp;
-    // CTAs per block: while the blocks leave half of the SMs idle, clusters of 2, 4 or 8 CTAs
-    // split a block's tiles (at least two tiles each at the longest length). A cluster's CTAs sit
-    // in one GPC, which leaves some of its SMs over: pairs fill all of them, clusters of 4 and 8
-    // are counted on for 27/32. (6 sequences of 46000 tokens, 112-token chunks, 12 heads, 72
-    // blocks: 379 us, in pairs 219.)
-    const int64_t blocks = blocks_of(la.hp) * g.Hkv * g.B;
-    const int64_t tiles = ((int64_t)g.max_pages * g.P + kBN - 1) / kBN;
-    while (la.cs < 8 && la.cs * 4 <= tiles &&
-           blocks * la.cs * 2 * 32 <= (int64_t)device_sm_count() * (la.cs == 1 ? 32 : 27))
-        la.cs *= 2;
+    const PrefillPlan plan = plan_prefill(g.B, g.Hkv, g.G, a.max_q, (int64_t)g.max_pages * g.P,
+                                          g.wr_per_qh != 0, device_sm_count());
+    la.hp = plan.hp;
+    la.rpb = plan.rpb;
+    la.cs = plan.cs;
     CUtensorMap vmap, wmap, qmap;
     {
         // cache as [num_pages * Hkv * P rows][128], one box = one page of one head (64 dims)
