@@ -14,10 +14,12 @@
 //    meet only at the end, where their two states are merged like two splits.
 //  NG = 1, two CTAs per SM with a ring of 3 tiles, 16 heads: for launches of several waves, whose
 //    start-ups and last wave then overlap and share HBM.
-// The output MMAs of kFold tiles accumulate in TMEM; then the group adds that sum to its O (fp32
-// columns in TMEM, rounded to nearest by the compute warps) and the next tile starts it over.
-// (Left to the MMAs for a whole run, the tensor core's truncating adds raised the fp32 output's
-// error against 64 bits from 2.5e-6 to 4.8e-6 at 8192 tokens.) The rare tile that moves a
+// After each tile the group adds the MMAs' O to its sum (fp32 columns in TMEM, rounded to nearest by
+// the compute warps) and the next tile's MMAs start over, as the sibling CTAs do it: the tensor core's
+// adds truncate. (fp32 outputs against 64 bits, 32 sequences of 300 to 8000 tokens, 128/8 heads:
+// 2.65e-6, siblings 2.64e-6; with the MMAs adding up 4 tiles of a group 2.70e-6, a whole run 4.8e-6
+// at 8192 tokens. Folding every tile instead of every fourth costs 1 to 3 %: 256 sequences of 32/1
+// heads 105.3 -> 106.9 us, 64 of 1000 to 60000 tokens 173.5 -> 178.7.) The rare tile that moves a
 // reference rescales both.
 //
 // Warps: group i = warps 8 i .. 8 i + 7: warp w of a group reads TMEM lane quarter w % 4 (thread =
@@ -41,7 +43,6 @@ namespace {
 
 constexpr int kWideGroupThreads = 256;               // 8 compute warps per softmax group
 constexpr uint32_t kBarGroup = 3;                    // + group: vote of one group's warps
-constexpr int kFold = 4;                             // tiles of a group summed by the MMAs alone
 constexpr int kWideMaxRuns = 256;                    // states merged per (b, g, head block)
 // A reference moves when a weight 2^(s - m) passes this. Sums, O and the split-bf16 weights are
 // floating point with fp32's exponent range, so a stale reference costs no precision; the bound
@@ -173,8 +174,8 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
     constexpr int N = 2 * NH;                            // MMA columns: hi | lo
     constexpr uint32_t kQHalf = N * 128;                 // one 64-dim half of the query operand
     constexpr uint32_t kGroupBytes = N / 8 * 128;        // P: one group of 8 tokens
-    // TMEM columns: two S buffers and the MMAs' sum O of each group, N each; then each group's
-    // folded O, NH each
+    // TMEM columns: two S buffers and the O of a tile of each group, N each; then each group's summed
+    // O, NH each
     constexpr uint32_t kColS = 0, kColO = 2 * NG * N, kColF = 3 * NG * N;
     static_assert(kColF + NG * NH <= kWideTmemCols, "");
     // (aligned by declaration: with two CTAs per SM there is no room for slack)
@@ -447,7 +448,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
                 const uint64_t b0 = p_desc + ((pb * sizeof(sm.p[0])) >> 4);
                 for (int kk = 0; kk < ksteps; ++kk)
                     ptx::mma_bf16(tmem + kColO + pb * N, a0 + ((kk * 2048) >> 4),
-                                  b0 + ((kk * 2 * kGroupBytes) >> 4), idesc_o, k % kFold != 0 || kk > 0);
+                                  b0 + ((kk * 2 * kGroupBytes) >> 4), idesc_o, kk > 0);
                 ptx::mma_commit(&sm.o_full[pb]);
                 ptx::mma_commit(&sm.empty[s]);
             }
@@ -516,7 +517,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
         // One barrier per tile for the group: it counts the threads with a weight past the slack
         // or a failed wait. Only then a second one exchanges the tile maxima (or lets the whole
         // group leave together).
-        // folded O of heads h .. h + 7 += the MMAs' sum, hi and lo (thread = output dim t)
+        // summed O of heads h .. h + 7 += the tile's O, hi and lo (thread = output dim t)
         auto fold = [&](int h, bool add) {
             float oh[8], ol[8];
             const uint32_t oc = tmem + kColO + grp * N + h + lane_base;
@@ -598,7 +599,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
                         p[c + e] = ptx::ex2(p[c + e] - mn);
                     }
                     if (!first) {
-                        // O holds the group's earlier tiles: rescale it in TMEM
+                        // O holds the group's previous tile, the sum the ones before it: rescale both
                         float oh[8], ol[8];
                         const uint32_t oc = tmem + kColO + grp * N + h0 + c + lane_base;
                         tmem_ld_cols8(oc, oc + NH, oh, ol);
@@ -609,7 +610,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
                         }
                         tmem_st_cols8(oc, oh);
                         tmem_st_cols8(oc + NH, ol);
-                        if (k > kFold) {
+                        if (k > 1) {
                             const uint32_t fc = tmem + kColF + grp * NH + h0 + c + lane_base;
                             tmem_ld_col8(fc, oh);
 #pragma unroll
@@ -649,11 +650,11 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
             }
             if (!freed) carried = wait(&sm.o_full[grp], (k - 1) & 1);
             if (carried) {
-                if (k % kFold == 0 && k > 0) {
-                    // fold the MMAs' sum of the last kFold tiles; this tile's MMAs start it over
+                if (k > 0) {
+                    // fold the group's previous tile; this tile's MMAs start over
                     ptx::tc_fence_after();
 #pragma unroll
-                    for (int c = 0; c < KH; c += 8) fold(h0 + c, k > kFold);
+                    for (int c = 0; c < KH; c += 8) fold(h0 + c, k > 1);
                     ptx::tmem_wait_st();
                     ptx::tc_fence_before();
                 }
@@ -703,8 +704,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
             const bool write_out = a.direct_out || n_cta_u == 1;
             const bool two = NG == 2 && n_tiles > 1;
             const int mine0 = (n_tiles + NG - 1) / NG;
-            // O of heads h1 .. h1 + KR - 1 of a group that ran n tiles: the folded sum and the MMAs'
-            // last one
+            // O of heads h1 .. h1 + KR - 1 of a group that ran n tiles: the sum and the last tile's
             auto group_o = [&](int gi, int n, float (&o)[KR]) {
                 const uint32_t oc = tmem + kColO + gi * N + h1 + lane_base;
                 const uint32_t fc = tmem + kColF + gi * NH + h1 + lane_base;
@@ -713,7 +713,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
                     tmem_ld_cols8(oc, oc + NH, o, lo);
 #pragma unroll
                     for (int e = 0; e < 8; ++e) o[e] += lo[e];
-                    if (n > kFold) {
+                    if (n > 1) {
                         tmem_ld_col8(fc, lo);
 #pragma unroll
                         for (int e = 0; e < 8; ++e) o[e] += lo[e];
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
 #pragma unroll
                     for (int e = 0; e < KR; ++e) {
                         o[e] = ptx::tmem_ld1(oc + e) + ptx::tmem_ld1(oc + NH + e);
-                        if (n > kFold) o[e] += ptx::tmem_ld1(fc + e);
+                        if (n > 1) o[e] += ptx::tmem_ld1(fc + e);
                     }
                 }
             };
