@@ -48,7 +48,11 @@
 // routed query is scaled before its bf16 rounding), so p = 2^(s - m). The reference maximum m of
 // a row only moves when the tile maximum exceeds it by more than 8 (a factor 256): then the row's
 // O in TMEM and its running sum l are rescaled; otherwise p may reach 2^8, well inside fp16 and
-// fp32 range, and the final O / l is unchanged because O and l share the same reference.
+// fp32 range, and the final O / l is unchanged because O and l share the same reference. The first
+// reference covers the first 128 tokens (two half tiles, one of each softmax group): the row's largest
+// weight is then more often exactly 1 and free of rounding. (With the first 64 alone fp32 outputs
+// were further off from 64 bits: rms 1.56e-4 instead of 1.49e-4 on rows of 200 tokens, 1.060e-4
+// instead of 1.044e-4 on a 4096-token prompt.)
 //
 // Roles (352 threads, one CTA per SM):
 //   warps 0-7  softmax and epilogue: warp w serves TMEM lane quarter w % 4 (its 32 query rows)
@@ -103,9 +107,11 @@ struct __align__(1024) PrefillSmem {
     uint64_t full[kStages], empty[kStages];
     uint64_t s_full[kSub], s_free[kSub], p_full[kSub];
     uint64_t turn[4][2];       // per lane quarter and parity: the references after a half tile
+    uint64_t first[4];         // per lane quarter: the maxima of half tile 1 are in lsum[1]
     uint64_t r_full, qr_ready, drain, drain2;
     float mref[2][kBM];        // the rows' references after the last half tile of each parity
-    float lsum[2][kBM];        // the two groups' shares of the row sums, for the epilogue
+    float lsum[2][kBM];        // the two groups' shares of the row sums, for the epilogue (before:
+                               // [1] the maxima of half tile 1, for the first reference)
     float2 ml[kBM];            // the rows' references and sums, for the cluster's merge
     uint32_t tmem_base;
     int abort;
@@ -268,8 +274,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             ptx::mbar_init(&sm.s_free[b2], 1);
             ptx::mbar_init(&sm.p_full[b2], kComputeWarps / 2);
         }
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 4; ++q) {
             for (int b2 = 0; b2 < 2; ++b2) ptx::mbar_init(&sm.turn[q][b2], 1);
+            ptx::mbar_init(&sm.first[q], 1);
+        }
         ptx::mbar_init(&sm.r_full, 1);
         ptx::mbar_init(&sm.qr_ready, kComputeWarps);
         ptx::mbar_init(&sm.drain, 1);
@@ -536,9 +544,21 @@ __global__ void __launch_bounds__(kThreads, 1)
                 mx[2] = max3(mx[2], __uint_as_float(s1[c]), __uint_as_float(s1[c + 1]));
                 mx[3] = max3(mx[3], __uint_as_float(s1[c + 2]), __uint_as_float(s1[c + 3]));
             }
-            const float mt = max3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
+            float mt = max3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
             float m_ref = -INFINITY;
-            if (u > 0) {
+            if (u == 0) {
+                // the row's first reference is the maximum of its first two half tiles
+                if (n_sub > 1) {
+                    okl = wait(&sm.first[qd], 0);
+                    if (!okl) break;
+                    mt = fmaxf(mt, sm.lsum[1][r]);
+                }
+            } else {
+                if (u == 1) {
+                    sm.lsum[1][r] = mt;
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&sm.first[qd]);
+                }
                 okl = wait(&sm.turn[qd][hf ^ 1], ((u - 1) >> 1) & 1);
                 if (!okl) break;
                 m_ref = sm.mref[hf ^ 1][r];
