@@ -46,13 +46,16 @@
 //
 // Softmax (thread = query row = TMEM lane): scores arrive already scaled by scale * log2 e (the
 // routed query is scaled before its bf16 rounding), so p = 2^(s - m). The reference maximum m of
-// a row only moves when the tile maximum exceeds it by more than 8 (a factor 256): then the row's
-// O in TMEM and its running sum l are rescaled; otherwise p may reach 2^8, well inside fp16 and
+// a row only moves when a half tile's maximum exceeds it by more than 7 (a factor 128): then the row's
+// O in TMEM and its running sum l are rescaled; otherwise p may reach 2^7, well inside fp16 and
 // fp32 range, and the final O / l is unchanged because O and l share the same reference. The first
 // reference covers the first 128 tokens (two half tiles, one of each softmax group): the row's largest
 // weight is then more often exactly 1 and free of rounding. (With the first 64 alone fp32 outputs
 // were further off from 64 bits: rms 1.56e-4 instead of 1.49e-4 on rows of 200 tokens, 1.060e-4
-// instead of 1.044e-4 on a 4096-token prompt.)
+// instead of 1.044e-4 on a 4096-token prompt.) A reference that moves within a tile sees only its half
+// of the tile, so with the limit of 8 that suits whole tiles rows with outlier values were further
+// off as well, 1.19e-4 against 1.12e-4 (100-token chunks on 200 to 2000 tokens); with 7 they are at
+// 1.09e-4, for 1 to 2 % of the time of such inputs (4 x 512 rows on 4096 tokens 187 -> 191 us).
 //
 // Roles (352 threads, one CTA per SM):
 //   warps 0-7  softmax and epilogue: warp w serves TMEM lane quarter w % 4 (its 32 query rows)
@@ -94,7 +97,7 @@ constexpr uint32_t kColS = 0;                     // S of half tile u: 64 (u % 4
 constexpr uint32_t kColO = 256;                   // O: columns 256 .. 383
 constexpr uint32_t kColQ = 384;                   // Q_hi: 384 .. 447, Q_lo: 448 .. 511
 constexpr uint32_t kLoCols = 64;                  // hi -> lo of a packed bf16 operand
-constexpr float kRescaleLog2 = 8.f;
+constexpr float kRescaleLog2 = 7.f;
 constexpr uint64_t kTimeoutNs = 1000000000ull;
 
 struct __align__(1024) PrefillSmem {
@@ -563,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (!okl) break;
                 m_ref = sm.mref[hf ^ 1][r];
             }
-            // a new reference when the maximum grew by more than 2^8 (or is the first finite)
+            // a new reference when the maximum grew by more than 2^7 (or is the first finite)
             const float m_new = fmaxf(m_ref, mt);
             if (__any_sync(0xffffffffu, m_new > m_ref + kRescaleLog2)) {
                 const float f = (m_new == -INFINITY || m_ref == -INFINITY) ? 0.f : ptx::ex2(m_ref - m_new);
