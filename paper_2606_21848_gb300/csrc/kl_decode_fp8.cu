@@ -720,8 +720,11 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int h = 4 * blk + k;
-                        const float mn = fmaxf(mref[h], fmaxf(fmaxf(sm.red[grp][0][h], sm.red[grp][1][h]),
+                        // (scores all -inf so far, as a row of a group's own first tile may be: weights
+                        // 0 against any reference, and the reference stays -inf)
+                        const float mx = fmaxf(mref[h], fmaxf(fmaxf(sm.red[grp][0][h], sm.red[grp][1][h]),
                                                               fmaxf(sm.red[grp][2][h], sm.red[grp][3][h])));
+                        const float mn = mx == -INFINITY ? 0.f : mx;
                         alpha[k] = ptx::ex2(mref[h] - mn);
                         p_k[h] = ptx::ex2(p_k[h] - mn);
                         lsum[h] *= alpha[k];

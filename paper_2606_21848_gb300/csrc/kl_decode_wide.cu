@@ -45,8 +45,10 @@ constexpr int kWideGroupThreads = 256;               // 8 compute warps per soft
 constexpr uint32_t kBarGroup = 3;                    // + group: vote of one group's warps
 constexpr int kWideMaxRuns = 256;                    // states merged per (b, g, head block)
 // A reference moves when a weight 2^(s - m) passes this. Sums, O and the split-bf16 weights are
-// floating point with fp32's exponent range, so a stale reference costs no precision; the bound
-// only keeps everything far from overflow.
+// floating point with fp32's exponent range, so the bound only keeps everything far from overflow. (Of
+// the precision a stale reference costs only the chance that the largest weight is exactly 1: with a
+// slack of 4 the fp32 error was 0.3 % smaller on two of nine inputs, the same on the others, and 64
+// sequences of 1000 to 60000 tokens with outliers took 231 instead of 180 us.)
 constexpr float kWideLazy = 1024.f;
 
 // Warp roles and sizes for NH heads per CTA and NG softmax groups: NG = 2, one CTA per SM; NG = 1,
@@ -593,7 +595,9 @@ __global__ void __launch_bounds__(Wide<NH, NG>::kThreads, Wide<NH, NG>::kCtas)
                         const int h = h0 + c + e;
                         const float tmax = fmaxf(fmaxf(sm.red[grp][0][h], sm.red[grp][1][h]),
                                                  fmaxf(sm.red[grp][2][h], sm.red[grp][3][h]));
-                        const float mn = fmaxf(mref[c + e], tmax);
+                        // (scores all -inf so far, as a row of a group's own first tile may be: weights
+                        // 0 against any reference, and the reference stays -inf)
+                        const float mx = fmaxf(mref[c + e], tmax), mn = mx == -INFINITY ? 0.f : mx;
                         alpha[e] = ptx::ex2(mref[c + e] - mn);    // 0 for the first tile
                         lsum[c + e] *= alpha[e];
                         p[c + e] = ptx::ex2(p[c + e] - mn);
