@@ -133,6 +133,7 @@ def _call():
         spec = importlib.util.spec_from_file_location("_keyless", _build.PYMOD, loader=loader)
         _native = importlib.util.module_from_spec(spec)
         loader.exec_module(_native)
+        _native.types(kl_shape, kl_latent_shape, kl_decode_options)
     return _native
 
 

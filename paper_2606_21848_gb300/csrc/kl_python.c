@@ -1,8 +1,9 @@
 /*
  * Argument marshalling of the Python binding (_lib.py) in C: one function per launching entry
  * point of libkeyless. An address argument is None, an int, or an object with data_ptr(); a shape or
- * options argument is the ctypes structure of _lib.py; the stream is None (torch's current
- * stream), an int, or an object with cuda_stream. Each returns the kl_status.
+ * options argument is the ctypes structure of _lib.py (types() takes the classes); an integer has
+ * __index__() or is a ctypes c_int32; the stream is None (torch's current stream), an int, or an object with
+ * cuda_stream. Other types are refused with ctypes' own exceptions. Each returns the kl_status.
  *
  * A small decode takes the GPU 6 to 8 us and the C call 2, while ctypes with a c_void_p object per
  * argument and torch.cuda.current_stream() took 15 us of host time in front of it, plain ints and
@@ -16,10 +17,17 @@
 #include "keyless.h"
 
 static PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream;
-static PyObject *g_argument_error;                        /* ctypes.ArgumentError */
+static PyObject *s_value, *s_as_parameter;
+static PyObject *g_argument_error, *g_cdata, *g_c_int, *g_sizeof;   /* ctypes: ArgumentError, _CData, c_int32, sizeof */
+static PyObject *g_shape, *g_latent, *g_options;          /* the structure classes (types()) */
 static PyObject *g_initialized, *g_get_device, *g_raw_stream, *g_current_stream;   /* torch */
 
+/* The int `v`, as ctypes takes it (bits past the 64th dropped). */
 static int to_u64(PyObject *v, uint64_t *out) {
+    if (!PyLong_Check(v)) {
+        PyErr_Format(PyExc_TypeError, "expected an int, got %.100s", Py_TYPE(v)->tp_name);
+        return 0;
+    }
     *out = PyLong_AsUnsignedLongLongMask(v);
     return !(*out == (uint64_t)-1 && PyErr_Occurred());
 }
@@ -35,7 +43,7 @@ static int get_addr(PyObject *o, void **out) {
     } else {
         PyObject *v = PyObject_CallMethodNoArgs(o, s_data_ptr);
         if (!v) return 0;
-        const int ok = to_u64(v, &x);
+        const int ok = v == Py_None || to_u64(v, &x);
         Py_DECREF(v);
         if (!ok) return 0;
     }
@@ -44,25 +52,74 @@ static int get_addr(PyObject *o, void **out) {
 }
 
 static int get_i32(PyObject *o, int32_t *out) {
-    if (!PyLong_Check(o)) {
+    if (PyIndex_Check(o)) {
+        const unsigned long v = PyLong_AsUnsignedLongMask(o);
+        if (v == (unsigned long)-1 && PyErr_Occurred()) return 0;
+        *out = (int32_t)v;
+        return 1;
+    }
+    const int is_c = PyObject_IsInstance(o, g_c_int);
+    if (is_c < 0) return 0;
+    PyObject *v = PyObject_GetAttr(o, is_c ? s_value : s_as_parameter);
+    if (!v) {
+        PyErr_Clear();
         PyErr_Format(g_argument_error, "expected an int, got %.100s", Py_TYPE(o)->tp_name);
         return 0;
     }
-    const unsigned long v = PyLong_AsUnsignedLongMask(o);
-    if (v == (unsigned long)-1 && PyErr_Occurred()) return 0;
-    *out = (int32_t)v;
+    int ok = !Py_EnterRecursiveCall(" in an integer argument");
+    if (ok) {
+        ok = get_i32(v, out);
+        Py_LeaveRecursiveCall();
+    }
+    Py_DECREF(v);
+    return ok;
+}
+
+/* The contents of an instance of the ctypes structure `type` (`size` bytes, or a subclass's more). */
+static int get_struct(PyObject *o, void *out, Py_ssize_t size, PyObject *type) {
+    Py_buffer b;
+    if (!type) {
+        PyErr_SetString(PyExc_RuntimeError, "types() first");
+        return 0;
+    }
+    int is = PyObject_IsInstance(o, type);
+    if (is == 0) {
+        is = PyObject_IsInstance(o, g_cdata);
+        if (is >= 0)
+            PyErr_Format(is ? g_argument_error : PyExc_TypeError, "expected %.100s, got %.100s",
+                         ((PyTypeObject *)type)->tp_name, Py_TYPE(o)->tp_name);
+        return 0;
+    }
+    if (is < 0 || PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) < 0) return 0;
+    memcpy(out, b.buf, (size_t)size);
+    PyBuffer_Release(&b);
     return 1;
 }
 
-/* The contents of a ctypes structure of exactly `size` bytes. */
-static int get_struct(PyObject *o, void *out, Py_ssize_t size) {
-    Py_buffer b;
-    if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) < 0) return 0;
-    const int ok = b.len == size;
-    if (ok) memcpy(out, b.buf, (size_t)size);
-    PyBuffer_Release(&b);
-    if (!ok) PyErr_SetString(g_argument_error, "a structure of another type");
-    return ok;
+/* types(shape, latent_shape, options): the structure classes that the functions take. */
+static PyObject *py_types(PyObject *m, PyObject *const *a, Py_ssize_t na) {
+    (void)m;
+    const Py_ssize_t size[3] = {sizeof(kl_shape), sizeof(kl_latent_shape), sizeof(kl_decode_options)};
+    PyObject **to[3] = {&g_shape, &g_latent, &g_options};
+    if (na != 3) {
+        PyErr_SetString(PyExc_TypeError, "types takes 3 arguments");
+        return NULL;
+    }
+    for (int i = 0; i < 3; ++i) {
+        PyObject *n = PyObject_CallOneArg(g_sizeof, a[i]);
+        if (!n) return NULL;
+        const Py_ssize_t have = PyLong_AsSsize_t(n);
+        Py_DECREF(n);
+        if (have != size[i] || !PyType_Check(a[i])) {
+            if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "a structure of another size");
+            return NULL;
+        }
+    }
+    for (int i = 0; i < 3; ++i) {
+        Py_INCREF(a[i]);
+        Py_XSETREF(*to[i], a[i]);
+    }
+    Py_RETURN_NONE;
 }
 
 /* numel() * element_size() of a tensor, 0 of None. */
@@ -105,7 +162,7 @@ static int get_stream(PyObject *o, kl_stream_t *out) {
     } else if (o != Py_None) {
         v = PyObject_GetAttr(o, s_cuda_stream);
         if (!v) return 0;
-        const int ok = to_u64(v, &x);
+        const int ok = v == Py_None || to_u64(v, &x);
         Py_DECREF(v);
         if (!ok) return 0;
     } else {
@@ -135,12 +192,12 @@ static int get_stream(PyObject *o, kl_stream_t *out) {
     return 1;
 }
 
-#define SHAPE(i) kl_shape sh; if (!get_struct(a[i], &sh, sizeof sh)) return NULL
-#define LATENT(i) kl_latent_shape sh; if (!get_struct(a[i], &sh, sizeof sh)) return NULL
+#define SHAPE(i) kl_shape sh; if (!get_struct(a[i], &sh, sizeof sh, g_shape)) return NULL
+#define LATENT(i) kl_latent_shape sh; if (!get_struct(a[i], &sh, sizeof sh, g_latent)) return NULL
 #define PTR(i, x) void *x; if (!get_addr(a[i], &x)) return NULL
 #define INT(i, x) int32_t x; if (!get_i32(a[i], &x)) return NULL
 #define OPTS(i) kl_decode_options o; const int has_o = a[i] != Py_None; \
-    if (has_o && !get_struct(a[i], &o, sizeof o)) return NULL
+    if (has_o && !get_struct(a[i], &o, sizeof o, g_options)) return NULL
 #define WORK(i) void *ws; size_t wsn; if (!get_addr(a[i], &ws) || !get_nbytes(a[i], &wsn)) return NULL
 #define STREAM(i) kl_stream_t st; if (!get_stream(a[i], &st)) return NULL
 #define FN(name, n) static PyObject *py_##name(PyObject *m, PyObject *const *a, Py_ssize_t na) { \
@@ -214,7 +271,8 @@ static PyMethodDef methods[] = {
     M(route_query), M(append_v), M(decode_attention), M(decode_attention_ex), M(decode_step), M(combine),
     M(standard_decode), M(decode_attention_noalloc), M(append_v_chunk), M(prefill_attention),
     M(append_v_fp8), M(quantize_cache_fp8), M(decode_attention_fp8), M(decode_step_fp8),
-    M(latent_decode), M(latent_decode_step), {NULL, NULL, 0, NULL}};
+    M(latent_decode), M(latent_decode_step),
+    {"types", (PyCFunction)(void (*)(void))py_types, METH_FASTCALL, NULL}, {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_keyless", NULL, -1, methods,
                                     NULL, NULL, NULL, NULL};
 
@@ -222,12 +280,19 @@ PyMODINIT_FUNC PyInit__keyless(void) {
     PyObject *c = PyImport_ImportModule("ctypes");
     if (!c) return NULL;
     g_argument_error = PyObject_GetAttrString(c, "ArgumentError");
+    g_c_int = PyObject_GetAttrString(c, "c_int32");
+    g_sizeof = PyObject_GetAttrString(c, "sizeof");
+    PyObject *st = PyObject_GetAttrString(c, "Structure");
+    g_cdata = st ? PyObject_GetAttrString(st, "__base__") : NULL;
+    Py_XDECREF(st);
     Py_DECREF(c);
-    if (!g_argument_error) return NULL;
+    if (!g_argument_error || !g_c_int || !g_sizeof || !g_cdata) return NULL;
     if (!(s_data_ptr = PyUnicode_InternFromString("data_ptr")) ||
         !(s_numel = PyUnicode_InternFromString("numel")) ||
         !(s_element_size = PyUnicode_InternFromString("element_size")) ||
-        !(s_cuda_stream = PyUnicode_InternFromString("cuda_stream")))
+        !(s_cuda_stream = PyUnicode_InternFromString("cuda_stream")) ||
+        !(s_value = PyUnicode_InternFromString("value")) ||
+        !(s_as_parameter = PyUnicode_InternFromString("_as_parameter_")))
         return NULL;
     return PyModule_Create(&module);
 }
