@@ -123,17 +123,20 @@ _native = None
 
 
 def _call():
-    """The marshalling module (csrc/kl_python.c), loaded next to the library."""
+    """The marshalling module (csrc/kl_python.c), bound to the library that load() gives."""
     global _native
     if _native is None:
-        load()
+        lib = load()
         if not os.path.exists(_build.PYMOD):
             raise RuntimeError(f"the binding is not built ({_build.PYMOD} missing); call build() first")
         loader = importlib.machinery.ExtensionFileLoader("_keyless", _build.PYMOD)
         spec = importlib.util.spec_from_file_location("_keyless", _build.PYMOD, loader=loader)
-        _native = importlib.util.module_from_spec(spec)
-        loader.exec_module(_native)
-        _native.types(kl_shape, kl_latent_shape, kl_decode_options)
+        module = importlib.util.module_from_spec(spec)
+        loader.exec_module(module)
+        entries = {n: ctypes.cast(getattr(lib, n), ctypes.c_void_p).value
+                   for n in dir(module) if n.startswith("kl_")}
+        module.bind(entries, kl_shape, kl_latent_shape, kl_decode_options)
+        _native = module
     return _native
 
 

@@ -74,11 +74,10 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | N
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
-    # the Python module beside it (host C, linked to the library in its own folder)
+    # the Python module beside it (host C; bound to the library at run time)
     tmp = PYMOD + ".tmp"
     cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", INCLUDE,
-           "-I", sysconfig.get_paths()["include"], PYSRC, "-o", tmp, "-L", BUILD, "-l:libkeyless.so",
-           "-Wl,-rpath,$ORIGIN"]
+           "-I", sysconfig.get_paths()["include"], PYSRC, "-o", tmp]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"building the Python module failed:\n{r.stdout}\n{r.stderr}")

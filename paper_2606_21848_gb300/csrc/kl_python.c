@@ -1,9 +1,13 @@
 /*
  * Argument marshalling of the Python binding (_lib.py) in C: one function per launching entry
  * point of libkeyless. An address argument is None, an int, or an object with data_ptr(); a shape or
- * options argument is the ctypes structure of _lib.py (types() takes the classes); an integer has
- * __index__() or is a ctypes c_int32; the stream is None (torch's current stream), an int, or an object with
- * cuda_stream. Other types are refused with ctypes' own exceptions. Each returns the kl_status.
+ * options argument is the ctypes structure of _lib.py; an integer has __index__() or is a ctypes
+ * c_int32; the stream is None (torch's current stream), an int, or an object with cuda_stream. Other
+ * types are refused with ctypes' own exceptions. Each returns the kl_status.
+ *
+ * The module is not linked to libkeyless: bind() takes the entry points' addresses from the library
+ * that _lib.py has loaded (and the structure classes), so that both always call the same copy, whatever
+ * the loader's search path holds.
  *
  * A small decode takes the GPU 6 to 8 us and the C call 2, while ctypes with a c_void_p object per
  * argument and torch.cuda.current_stream() took 15 us of host time in front of it, plain ints and
@@ -19,8 +23,19 @@
 static PyObject *s_data_ptr, *s_numel, *s_element_size, *s_cuda_stream;
 static PyObject *s_value, *s_as_parameter;
 static PyObject *g_argument_error, *g_cdata, *g_c_int, *g_sizeof;   /* ctypes: ArgumentError, _CData, c_int32, sizeof */
-static PyObject *g_shape, *g_latent, *g_options;          /* the structure classes (types()) */
+static PyObject *g_shape, *g_latent, *g_options;          /* the structure classes (bind()) */
 static PyObject *g_initialized, *g_get_device, *g_raw_stream, *g_current_stream;   /* torch */
+
+#define ENTRIES(X) \
+    X(route_query) X(append_v) X(decode_attention) X(decode_attention_ex) X(decode_step) X(combine) \
+    X(standard_decode) X(decode_attention_noalloc) X(append_v_chunk) X(prefill_attention) \
+    X(append_v_fp8) X(quantize_cache_fp8) X(decode_attention_fp8) X(decode_step_fp8) \
+    X(latent_decode) X(latent_decode_step)
+#define POINTER(n) static __typeof__(kl_##n) *f_##n;
+ENTRIES(POINTER)
+#define SLOT(n) {"kl_" #n, &f_##n},
+static const struct { const char *name; void *to; } slots[] = {ENTRIES(SLOT)};
+enum { kEntries = sizeof slots / sizeof slots[0] };
 
 /* The int `v`, as ctypes takes it (bits past the 64th dropped). */
 static int to_u64(PyObject *v, uint64_t *out) {
@@ -79,7 +94,7 @@ static int get_i32(PyObject *o, int32_t *out) {
 static int get_struct(PyObject *o, void *out, Py_ssize_t size, PyObject *type) {
     Py_buffer b;
     if (!type) {
-        PyErr_SetString(PyExc_RuntimeError, "types() first");
+        PyErr_SetString(PyExc_RuntimeError, "bind() first");
         return 0;
     }
     int is = PyObject_IsInstance(o, type);
@@ -96,28 +111,38 @@ static int get_struct(PyObject *o, void *out, Py_ssize_t size, PyObject *type) {
     return 1;
 }
 
-/* types(shape, latent_shape, options): the structure classes that the functions take. */
-static PyObject *py_types(PyObject *m, PyObject *const *a, Py_ssize_t na) {
+/* bind({name: address}, shape, latent_shape, options): the library's entry points and the structure
+ * classes that they take. */
+static PyObject *py_bind(PyObject *m, PyObject *const *a, Py_ssize_t na) {
     (void)m;
     const Py_ssize_t size[3] = {sizeof(kl_shape), sizeof(kl_latent_shape), sizeof(kl_decode_options)};
     PyObject **to[3] = {&g_shape, &g_latent, &g_options};
-    if (na != 3) {
-        PyErr_SetString(PyExc_TypeError, "types takes 3 arguments");
+    void *entry[kEntries];
+    if (na != 4 || !PyDict_Check(a[0])) {
+        PyErr_SetString(PyExc_TypeError, "bind takes a dict and 3 classes");
         return NULL;
     }
-    for (int i = 0; i < 3; ++i) {
-        PyObject *n = PyObject_CallOneArg(g_sizeof, a[i]);
-        if (!n) return NULL;
-        const Py_ssize_t have = PyLong_AsSsize_t(n);
-        Py_DECREF(n);
-        if (have != size[i] || !PyType_Check(a[i])) {
-            if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "a structure of another size");
+    for (int i = 0; i < kEntries; ++i) {
+        PyObject *v = PyDict_GetItemString(a[0], slots[i].name);
+        if (!v || !(entry[i] = PyLong_AsVoidPtr(v))) {
+            if (!PyErr_Occurred()) PyErr_SetString(PyExc_KeyError, slots[i].name);
             return NULL;
         }
     }
     for (int i = 0; i < 3; ++i) {
-        Py_INCREF(a[i]);
-        Py_XSETREF(*to[i], a[i]);
+        PyObject *n = PyObject_CallOneArg(g_sizeof, a[1 + i]);
+        if (!n) return NULL;
+        const Py_ssize_t have = PyLong_AsSsize_t(n);
+        Py_DECREF(n);
+        if (have != size[i] || !PyType_Check(a[1 + i])) {
+            if (!PyErr_Occurred()) PyErr_SetString(PyExc_TypeError, "a structure of another size");
+            return NULL;
+        }
+    }
+    for (int i = 0; i < kEntries; ++i) memcpy(slots[i].to, &entry[i], sizeof(void *));
+    for (int i = 0; i < 3; ++i) {
+        Py_INCREF(a[1 + i]);
+        Py_XSETREF(*to[i], a[1 + i]);
     }
     Py_RETURN_NONE;
 }
@@ -207,72 +232,68 @@ static int get_stream(PyObject *o, kl_stream_t *out) {
     return PyLong_FromLong((long)r); }
 
 FN(route_query, 5) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, out); STREAM(4);
-CALL(kl_route_query(&sh, q, w, out, st))
+CALL(f_route_query(&sh, q, w, out, st))
 
 FN(append_v, 7) SHAPE(0); PTR(1, v); PTR(2, bt); PTR(3, pos); PTR(4, c); PTR(5, e); STREAM(6);
-CALL(kl_append_v(&sh, v, bt, pos, c, e, st))
+CALL(f_append_v(&sh, v, bt, pos, c, e, st))
 
 FN(decode_attention, 12) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl); INT(6, ns);
 PTR(7, out); INT(8, dt); WORK(9); PTR(10, e); STREAM(11);
-CALL(kl_decode_attention(&sh, q, w, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_decode_attention(&sh, q, w, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(decode_attention_ex, 12) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl); OPTS(6);
 PTR(7, out); INT(8, dt); WORK(9); PTR(10, e); STREAM(11);
-CALL(kl_decode_attention_ex(&sh, q, w, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_decode_attention_ex(&sh, q, w, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(decode_step, 14) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, v); PTR(4, pos); PTR(5, c); PTR(6, bt);
 PTR(7, sl); OPTS(8); PTR(9, out); INT(10, dt); WORK(11); PTR(12, e); STREAM(13);
-CALL(kl_decode_step(&sh, q, w, v, pos, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_decode_step(&sh, q, w, v, pos, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(combine, 7) SHAPE(0); PTR(1, po); PTR(2, ml); INT(3, ns); PTR(4, out); INT(5, dt); STREAM(6);
-CALL(kl_combine(&sh, po, ml, ns, out, (kl_dtype)dt, st))
+CALL(f_combine(&sh, po, ml, ns, out, (kl_dtype)dt, st))
 
 FN(standard_decode, 12) SHAPE(0); PTR(1, q); PTR(2, k); PTR(3, c); PTR(4, bt); PTR(5, sl); OPTS(6);
 PTR(7, out); INT(8, dt); WORK(9); PTR(10, e); STREAM(11);
-CALL(kl_standard_decode(&sh, q, k, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_standard_decode(&sh, q, k, c, bt, sl, has_o ? &o : NULL, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(decode_attention_noalloc, 11) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl);
 INT(6, ns); PTR(7, out); INT(8, dt); PTR(9, e); STREAM(10);
-CALL(kl_decode_attention_noalloc(&sh, q, w, c, bt, sl, ns, out, (kl_dtype)dt, e, st))
+CALL(f_decode_attention_noalloc(&sh, q, w, c, bt, sl, ns, out, (kl_dtype)dt, e, st))
 
 FN(append_v_chunk, 10) SHAPE(0); PTR(1, v); PTR(2, bt); PTR(3, sl); PTR(4, cu); INT(5, tq); INT(6, mq);
 PTR(7, c); PTR(8, e); STREAM(9);
-CALL(kl_append_v_chunk(&sh, v, bt, sl, cu, tq, mq, c, e, st))
+CALL(f_append_v_chunk(&sh, v, bt, sl, cu, tq, mq, c, e, st))
 
 FN(prefill_attention, 13) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, bt); PTR(5, sl); PTR(6, cu);
 INT(7, tq); INT(8, mq); PTR(9, out); INT(10, dt); PTR(11, e); STREAM(12);
-CALL(kl_prefill_attention(&sh, q, w, c, bt, sl, cu, tq, mq, out, (kl_dtype)dt, e, st))
+CALL(f_prefill_attention(&sh, q, w, c, bt, sl, cu, tq, mq, out, (kl_dtype)dt, e, st))
 
 FN(append_v_fp8, 8) SHAPE(0); PTR(1, v); PTR(2, bt); PTR(3, pos); PTR(4, c); PTR(5, s); PTR(6, e);
 STREAM(7);
-CALL(kl_append_v_fp8(&sh, v, bt, pos, c, s, e, st))
+CALL(f_append_v_fp8(&sh, v, bt, pos, c, s, e, st))
 
 FN(quantize_cache_fp8, 5) SHAPE(0); PTR(1, v); PTR(2, c); PTR(3, s); STREAM(4);
-CALL(kl_quantize_cache_fp8(&sh, v, c, s, st))
+CALL(f_quantize_cache_fp8(&sh, v, c, s, st))
 
 FN(decode_attention_fp8, 13) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, c); PTR(4, s); PTR(5, bt); PTR(6, sl);
 INT(7, ns); PTR(8, out); INT(9, dt); WORK(10); PTR(11, e); STREAM(12);
-CALL(kl_decode_attention_fp8(&sh, q, w, c, s, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_decode_attention_fp8(&sh, q, w, c, s, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(decode_step_fp8, 15) SHAPE(0); PTR(1, q); PTR(2, w); PTR(3, v); PTR(4, pos); PTR(5, c); PTR(6, s);
 PTR(7, bt); PTR(8, sl); INT(9, ns); PTR(10, out); INT(11, dt); WORK(12); PTR(13, e); STREAM(14);
-CALL(kl_decode_step_fp8(&sh, q, w, v, pos, c, s, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_decode_step_fp8(&sh, q, w, v, pos, c, s, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(latent_decode, 13) LATENT(0); PTR(1, q); PTR(2, w); PTR(3, wp); PTR(4, c); PTR(5, bt); PTR(6, sl);
 INT(7, ns); PTR(8, out); INT(9, dt); WORK(10); PTR(11, e); STREAM(12);
-CALL(kl_latent_decode(&sh, q, w, wp, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_latent_decode(&sh, q, w, wp, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
 
 FN(latent_decode_step, 15) LATENT(0); PTR(1, q); PTR(2, w); PTR(3, wp); PTR(4, v); PTR(5, pos); PTR(6, c);
 PTR(7, bt); PTR(8, sl); INT(9, ns); PTR(10, out); INT(11, dt); WORK(12); PTR(13, e); STREAM(14);
-CALL(kl_latent_decode_step(&sh, q, w, wp, v, pos, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
+CALL(f_latent_decode_step(&sh, q, w, wp, v, pos, c, bt, sl, ns, out, (kl_dtype)dt, ws, wsn, e, st))
 
-#define M(name) {"kl_" #name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL}
+#define M(name) {"kl_" #name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, NULL},
 static PyMethodDef methods[] = {
-    M(route_query), M(append_v), M(decode_attention), M(decode_attention_ex), M(decode_step), M(combine),
-    M(standard_decode), M(decode_attention_noalloc), M(append_v_chunk), M(prefill_attention),
-    M(append_v_fp8), M(quantize_cache_fp8), M(decode_attention_fp8), M(decode_step_fp8),
-    M(latent_decode), M(latent_decode_step),
-    {"types", (PyCFunction)(void (*)(void))py_types, METH_FASTCALL, NULL}, {NULL, NULL, 0, NULL}};
+    ENTRIES(M) {"bind", (PyCFunction)(void (*)(void))py_bind, METH_FASTCALL, NULL}, {NULL, NULL, 0, NULL}};
 static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_keyless", NULL, -1, methods,
                                     NULL, NULL, NULL, NULL};
 
