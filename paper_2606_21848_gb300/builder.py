@@ -3,8 +3,8 @@
 Each translation unit under ``csrc/`` is compiled in parallel to an object file, then the
 objects are linked into ``_build/libkeyless.so`` with the CUDA runtime linked statically, so
 the library has no dependency beyond the driver; the binding's C module
-(``csrc/kl_python.c``) is compiled next to it. Rebuilds only when a source is newer than
-the library.
+(``csrc/kl_python.c``) is compiled next to it, for the interpreter that builds it. Each of the
+two is rebuilt only when one of its own sources is newer.
 """
 from __future__ import annotations
 
@@ -22,7 +22,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libkeyless.so")
 PYSRC = os.path.join(CSRC, "kl_python.c")
-PYMOD = os.path.join(BUILD, "_keyless.so")
+# named for the interpreter, as extension modules are: another Python builds its own beside it
+PYMOD = os.path.join(BUILD, "_keyless" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
@@ -40,18 +41,22 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(PYMOD):
-        return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(PYMOD))
-    deps = sources() + [PYSRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
-    return any(os.path.getmtime(p) > t for p in deps)
+def _stale(target: str, deps: list[str]) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in deps)
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | None = None) -> str:
-    """Compile every CUDA source for sm_103a and link libkeyless.so; returns its path."""
-    if not force and not _stale():
-        return LIB
+    """Build what is out of date: libkeyless.so for sm_103a (its path is returned) and the Python module."""
+    headers = glob.glob(os.path.join(INCLUDE, "*.h"))
+    if force or _stale(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + headers):
+        _build_library(verbose, extra_flags)
+    if force or _stale(PYMOD, [PYSRC] + headers):
+        _build_module()
+    return LIB
+
+
+def _build_library(verbose: bool, extra_flags: list[str] | None) -> None:
+    """Compile every CUDA source for sm_103a and link libkeyless.so."""
     os.makedirs(BUILD, exist_ok=True)
     cc = nvcc()
     flags = NVCC_FLAGS + (extra_flags or [])
@@ -74,7 +79,11 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | N
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, LIB)
-    # the Python module beside it (host C; bound to the library at run time)
+
+
+def _build_module() -> None:
+    """The binding's Python module (host C; bound to the library at run time)."""
+    os.makedirs(BUILD, exist_ok=True)
     tmp = PYMOD + ".tmp"
     cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", INCLUDE,
            "-I", sysconfig.get_paths()["include"], PYSRC, "-o", tmp]
@@ -82,7 +91,6 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | N
     if r.returncode != 0:
         raise RuntimeError(f"building the Python module failed:\n{r.stdout}\n{r.stderr}")
     os.replace(tmp, PYMOD)
-    return LIB
 
 
 if __name__ == "__main__":
