@@ -3,9 +3,9 @@
 Every function has the C name and the C argument order; tensors are passed as torch CUDA
 tensors (or raw device addresses as ints) and the stream defaults to torch's current stream.
 The launching functions go through a small C module (csrc/kl_python.c), the others and the
-structures through ctypes.
-A non-OK status raises :class:`KLError`. There is no fallback: if the library has not been
-built, :func:`load` raises.
+structures through ctypes; where Python's C headers are missing and the module cannot be built, the
+launching functions go through ctypes too.
+A non-OK status raises :class:`KLError`. If the library has not been built, :func:`load` raises.
 """
 from __future__ import annotations
 
@@ -122,12 +122,54 @@ def status_string(status: int) -> str:
 _native = None
 
 
+class _Ctypes:
+    """The module's functions through ctypes (15 us of host time per call instead of 2)."""
+
+    @staticmethod
+    def _address(x):
+        return ctypes.c_void_p(x if x is None or isinstance(x, int) else x.data_ptr())
+
+    @staticmethod
+    def _stream(x):
+        if x is None:
+            import torch
+            x = torch.cuda.current_stream()
+        return ctypes.c_void_p(x if isinstance(x, int) else x.cuda_stream)
+
+    def __getattr__(self, name):
+        f = getattr(load(), name)
+        last = len(f.argtypes) - 1
+
+        def call(*args):
+            given, out = iter(args), []
+            for i, t in enumerate(f.argtypes):
+                if t is ctypes.c_size_t:                  # the size of the workspace just before it
+                    out.append(0 if x is None else x.numel() * x.element_size())
+                    continue
+                x = next(given)
+                if i == last:
+                    out.append(self._stream(x))
+                elif t is ctypes.c_void_p:
+                    out.append(self._address(x))
+                elif t is ctypes.c_int32 or (x is None and t is ctypes.POINTER(kl_decode_options)):
+                    out.append(x)
+                else:
+                    out.append(ctypes.byref(x))
+            return f(*out)
+
+        setattr(self, name, call)
+        return call
+
+
 def _call():
     """The marshalling module (csrc/kl_python.c), bound to the library that load() gives."""
     global _native
     if _native is None:
         lib = load()
         if not os.path.exists(_build.PYMOD):
+            if _build.python_headers() is None:
+                _native = _Ctypes()
+                return _native
             raise RuntimeError(f"the binding is not built ({_build.PYMOD} missing); call build() first")
         loader = importlib.machinery.ExtensionFileLoader("_keyless", _build.PYMOD)
         spec = importlib.util.spec_from_file_location("_keyless", _build.PYMOD, loader=loader)

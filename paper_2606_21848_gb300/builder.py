@@ -4,7 +4,8 @@ Each translation unit under ``csrc/`` is compiled in parallel to an object file,
 objects are linked into ``_build/libkeyless.so`` with the CUDA runtime linked statically, so
 the library has no dependency beyond the driver; the binding's C module
 (``csrc/kl_python.c``) is compiled next to it, for the interpreter that builds it. Each of the
-two is rebuilt only when one of its own sources is newer.
+two is rebuilt only when one of its own sources is newer. Without Python's C headers the module is
+left out (and the binding goes through ctypes).
 """
 from __future__ import annotations
 
@@ -41,6 +42,15 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def python_headers() -> str | None:
+    """The folder of Python.h, or None where Python's C headers are not installed."""
+    paths = sysconfig.get_paths()
+    for d in (paths["include"], paths["platinclude"]):
+        if os.path.exists(os.path.join(d, "Python.h")):
+            return d
+    return None
+
+
 def _stale(target: str, deps: list[str]) -> bool:
     return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in deps)
 
@@ -50,8 +60,9 @@ def build(force: bool = False, verbose: bool = False, extra_flags: list[str] | N
     headers = glob.glob(os.path.join(INCLUDE, "*.h"))
     if force or _stale(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + headers):
         _build_library(verbose, extra_flags)
-    if force or _stale(PYMOD, [PYSRC] + headers):
-        _build_module()
+    include = python_headers()
+    if include and (force or _stale(PYMOD, [PYSRC] + headers)):
+        _build_module(include)
     return LIB
 
 
@@ -81,12 +92,12 @@ def _build_library(verbose: bool, extra_flags: list[str] | None) -> None:
     os.replace(tmp, LIB)
 
 
-def _build_module() -> None:
+def _build_module(include: str) -> None:
     """The binding's Python module (host C; bound to the library at run time)."""
     os.makedirs(BUILD, exist_ok=True)
     tmp = PYMOD + ".tmp"
     cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", INCLUDE,
-           "-I", sysconfig.get_paths()["include"], PYSRC, "-o", tmp]
+           "-I", include, PYSRC, "-o", tmp]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"building the Python module failed:\n{r.stdout}\n{r.stderr}")
