@@ -19,7 +19,7 @@ template <bool kStandard>
 cudaError_t launch(const DecodeArgs &a) {
     // groups of more than 8 heads: wide CTAs of up to 32 heads, unless the caller takes the split
     // states (one per split) or the K+V comparison is asked for (64 sequences of 128/8 heads, 8192
-    // tokens: 252 us with sibling CTAs, 163 wide; 256 of 32/1 heads: 248 and 105)
+    // tokens: 252 us with sibling CTAs, 164 wide; 256 of 32/1 heads: 248 and 107)
     if (!kStandard && a.geo.nhb > 1 && a.geo.D == 128 && (a.direct_out || a.merge_inside))
         return launch_tc_wide(a);
     DecodeArgs la = a;

@@ -27,10 +27,10 @@
 // producer, the score-MMA issuer (TMEM owner) and the output-MMA issuer.
 //
 // Measured (back-to-back calls, 8192 tokens): 64 sequences of 128 heads over 8 value heads 252 us
-// with sibling CTAs of 8 heads, 185 with NG = 2, 163 with NG = 1 (HBM floor 158); 256 sequences of
-// 32 heads over one value head 248 us with siblings, 129 with NG = 1 (two CTAs per tile, bound by
-// the ring's round trip), 105 with NH = 32 and NG = 2 (floor 80; the rest is the last, partly
-// filled wave). One sequence of 100000 tokens, 128 / 8 heads: 47.9 us with NG = 1, 39.8 with
+// with sibling CTAs of 8 heads, 184 with NG = 2, 164 to 168 with NG = 1 (HBM floor 158); 256 sequences
+// of 32 heads over one value head 248 us with siblings, 133 with NG = 1 (two CTAs per tile, bound by
+// the ring's round trip), 107 with NH = 32 and NG = 2 (floor 80; the rest is the last, partly
+// filled wave). One sequence of 100000 tokens, 128 / 8 heads: 49.0 us with NG = 1, 40.6 with
 // NG = 2. Spills cost much, since the shared memory leaves next to no L1: 48 bytes more per thread
 // and tile took the second case from 121 to 158 us, so the references live in shared memory and
 // the weights are formed 8 heads at a time.
@@ -832,11 +832,12 @@ cudaError_t launch_tc_wide(const DecodeArgs &a) {
             while ((int64_t)((g.S + spc - 1) / spc) * units > slots) ++spc;
         return spc;
     };
-    // Groups of 17 or more heads: CTAs of 32 heads (1180 cycles per tile where HBM does not set the
-    // pace), unless CTAs of 16 (1010) have an SM each and not 6/5 as many splits to run.
-    // (Group of 32, measured with CTAs of 16 and of 32: 104 sequences of 8192 tokens 65.8 and 50.8 us,
-    // 77 64.7 and 49.0, 30 of 32768 in 4 splits 71.4 and 55.3, 150 of 1000 in a group of 24 14.8 and
-    // 13.6; 52 sequences of 8192, one CTA of 16 on each of 104 SMs, 38.5 and about 45.)
+    // Groups of 17 or more heads: CTAs of 32 heads (about 1200 cycles per tile where HBM does not set
+    // the pace), unless CTAs of 16 (about 1000) have an SM each and not 6/5 as many splits to run.
+    // (Group of 32, measured with CTAs of 16 and of 32: 104 sequences of 8192 tokens 67.7 and 51.4 us,
+    // 77 68.1 and 49.8, 30 of 32768 in 4 splits 72.6 and 55.5, 20 of 40000 in 5 71.1 and 53.0, 150 of
+    // 1000 in a group of 24 14.9 and 13.9; 52 sequences of 8192, one CTA of 16 on each of 104 SMs,
+    // 39.1 and about 45.)
     const int64_t seq_heads = (int64_t)g.B * g.Hkv;
     const int64_t units32 = seq_heads * ((g.G + 31) / 32), units16 = seq_heads * ((g.G + 15) / 16);
     const bool w32 = g.G > 16 && (units16 > sms || 6 * splits_per_cta(units32, sms) <=

@@ -28,8 +28,11 @@ struct Geometry {
     int S;             // split count
     int chunk;         // tokens per split (a multiple of 128)
     int spc = 1;       // splits per CTA of the tensor-core decode (consecutive, same (b, g))
-    int nhb = 1;       // CTAs per (run of splits, b, g): blocks of up to 8 query heads
-    int qbox = 8;      // query rows of one CTA: min(G, 8), or 2 G with two value heads
+    // CTAs per (run of splits, b, g) and query rows of one CTA: as resolved, blocks of up to 8 query
+    // heads (qbox: min(G, 8), or 2 G with two value heads), which the split plan and the workspace
+    // count on; the wide decode's launcher sets its own blocks of 16 or 32 and spc for them.
+    int nhb = 1;
+    int qbox = 8;
     int vpc = 1;       // value heads per CTA of the tensor-core decode: 2 at head dim 64 (the
                        // two heads' rows side by side in one 128-wide tile), else 1
 };

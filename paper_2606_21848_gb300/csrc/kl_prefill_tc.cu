@@ -28,8 +28,9 @@
 // exponentials, weights, output, about 2600 cycles) is spread over four in flight. With whole
 // tiles and two buffers that chain set the pace; so did the issuing threads, which are held until
 // their MMAs start and then paid warp-wide waits before the next ones: each issuer's loop now
-// runs in one elected lane. 32K-token prompt (12 heads) 3340 -> 2970 us, 512-token chunks on 8192
-// (8 x 32 heads) 600 -> 543 us; the issued MMAs, 1.5 times the useful ones, then run at 1.68
+// runs in one elected lane. 32K-token prompt (12 heads) 3335 -> 3000 us, 512-token chunks on 8192
+// (8 x 32 heads) 595 -> 543 us (whole tiles and half tiles timed in turn; single boxes give 2980 to
+// 3140 us for the prompt); the issued MMAs, 1.5 times the useful ones, then run at 1.58 to 1.66
 // PFLOP/s under the power cap, where cuBLAS sustains 1.73.
 //
 // Precision: the routed query (times scale * log2 e) is carried as a pair of bf16 operands,

@@ -196,8 +196,6 @@ __device__ __forceinline__ void bar_sync(uint32_t id, uint32_t count) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
-// Barrier `id` over `count` threads that also returns the AND of `v` over them, so that a
-// decision (e.g. to leave a loop) is taken by all of them together.
 // Barrier `id` over `count` threads that also returns how many of them passed v = true.
 __device__ __forceinline__ uint32_t bar_popc(uint32_t id, uint32_t count, bool v) {
     uint32_t r;
@@ -211,6 +209,8 @@ __device__ __forceinline__ uint32_t bar_popc(uint32_t id, uint32_t count, bool v
     return r;
 }
 
+// Barrier `id` over `count` threads that also returns the AND of `v` over them, so that a
+// decision (e.g. to leave a loop) is taken by all of them together.
 __device__ __forceinline__ bool bar_and(uint32_t id, uint32_t count, bool v) {
     uint32_t r;
     asm volatile(
