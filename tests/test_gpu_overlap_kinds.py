@@ -112,3 +112,59 @@ def test_chain_of_kinds(B, Hq, Hkv, L, order):
         assert torch.equal(a.view(torch.int16), b.view(torch.int16)), f"graph {i} {calls[i].__name__}"
     for a, b in zip((cache, codes, scales), state):
         assert torch.equal(a.view(torch.uint8), b.view(torch.uint8))
+
+
+@pytest.mark.parametrize("Hq, Hkv, splits", [(32, 8, 1), (32, 8, 3), (64, 4, 1), (64, 4, 4)])
+def test_copies_and_other_streams_between(Hq, Hkv, splits):
+    """Between the calls a copy, a memset or another stream's kernel behind an event: what stands ahead
+    of a call in its stream is not a kernel, or more than one thing, and still comes first."""
+    B, D, P, L, steps = 6, 128, 16, 1100, 16
+    dev = _gpu.dev()
+    x = tiny(B=B, Hq=Hq, Hkv=Hkv, D=D, P=P, lens=(L, 40, 700, 1, 300, L), seed=280)
+    g = to_dev(x)
+    sh = kl.make_shape(B, Hq, Hkv, D, P, x["v_cache"].shape[0], x["block_table"].shape[1])
+    ws = torch.zeros(max(256, kl.kl_decode_workspace_size(sh, splits)), dtype=torch.uint8, device=dev)
+    err = torch.zeros(1, dtype=torch.int32, device=dev)
+    q = [torch.empty_like(g["q"]) for _ in range(steps + 1)]
+    out = [torch.empty_like(g["q"]) for _ in range(steps)]
+    side = torch.cuda.Stream()
+    v_new = g["v_new"]
+
+    def run(sync):
+        q[0].copy_(g["q"])
+        main = torch.cuda.current_stream()
+        for i in range(steps):
+            kl.kl_append_v(sh, v_new, g["block_table"], g["positions"], g["v_cache"], err)
+            kl.kl_decode_attention(sh, q[i], g["w_r"], g["v_cache"], g["block_table"], g["seq_lens"], splits,
+                                   out[i], kl.KL_BF16, ws, err)
+            if i % 3 == 0:                              # a copy of the result, on the same stream
+                q[i + 1].copy_(out[i])
+            elif i % 3 == 1:                            # another stream makes the next query
+                side.wait_stream(main)
+                with torch.cuda.stream(side):
+                    q[i + 1].copy_(out[i]).mul_(1.5)
+                main.wait_stream(side)
+            else:                                       # a memset, then a kernel
+                q[i + 1].zero_()
+                q[i + 1].add_(out[i])
+            if sync:
+                torch.cuda.synchronize()
+
+    run(True)
+    want = [b.clone() for b in out]
+    for b in out + q:
+        b.fill_(float("nan"))
+    run(False)
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    for i, (a, b) in enumerate(zip(out, want)):
+        assert torch.isfinite(b).all() and torch.equal(a.view(torch.int16), b.view(torch.int16)), i
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        run(False)
+    for b in out + q:
+        b.fill_(float("nan"))
+    graph.replay()
+    torch.cuda.synchronize()
+    for i, (a, b) in enumerate(zip(out, want)):
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16)), f"graph {i}"
