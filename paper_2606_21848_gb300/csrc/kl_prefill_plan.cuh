@@ -37,7 +37,7 @@ inline PrefillPlan plan_prefill(int B, int Hkv, int G, int max_q, int64_t max_to
     // split a block's tiles (at least two tiles each at the longest length). A cluster's CTAs sit
     // in one GPC, which leaves some of its SMs over: pairs fill all of them, clusters of 4 and 8
     // are counted on for 27/32. (6 sequences of 46000 tokens, 112-token chunks, 12 heads, 72
-    // blocks: 379 us, in pairs 219.)
+    // blocks: 379 us, in pairs 207.)
     const int64_t blocks = blocks_of(p.hp) * Hkv * B;
     const int64_t tiles = (max_tokens + kPrefillTile - 1) / kPrefillTile;
     while (p.cs < 8 && p.cs * 4 <= tiles && blocks * p.cs * 2 * 32 <= (int64_t)sms * (p.cs == 1 ? 32 : 27))

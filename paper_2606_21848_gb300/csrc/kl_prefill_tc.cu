@@ -6,8 +6,9 @@
 // cached rows), so the CTA walks the cache tiles 0 .. p_last / 128 and masks only the last ones.
 // Small chunks share more (kShared): a block's 128 rows hold several heads of a group, which read
 // the same tiles, and while the blocks leave SMs idle, a cluster of up to 8 CTAs splits a block's
-// tiles and merges the states through distributed shared memory. (4 sequences of 4000 tokens,
-// 16-token chunks, 12 heads: 43 -> 27 us; 2 of 8000 tokens, 100-token chunks, 32 heads: 85 -> 56.)
+// tiles and merges the states through distributed shared memory. (Chunk append and prefill, back to
+// back: 4 sequences of 4000 tokens, 16-token chunks, 12 heads: 52 -> 17 us; 2 of 8000 tokens, 100-token
+// chunks, 32 heads: 93 -> 51.)
 //
 //   routing  Q_r = Q . W^R[w(h)]                      M = 128 rows, N = 128, K = 128 (Section 2.2)
 //   scores   S   = Q_hi . V_t^T + Q_lo . V_t^T        M = 128 rows, N = 128 tokens, K = 2 x 128
